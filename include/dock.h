@@ -101,7 +101,9 @@ typedef struct {
   float clash_dist;           /* bump threshold d_c (Angstrom): a pair closer than d_c bumps */
   int32_t post_align;         /* 1: repeat the rigid alignment after the torsion sweep */
   int32_t early_exit;         /* 1: stop testing an angle's pairs at its first bump and skip
-                                 scoring rejected angles (results are identical either way) */
+                                 scoring rejected angles, and in the rigid alignment on a trilinear grid
+                                 score only the poses that an estimate with a proved error bound leaves
+                                 in the running (results are identical either way) */
   uint64_t seed;              /* keys the restart orientations together with the ligand id */
   int32_t select_k;           /* Select Poses (Alg. 1, after the restart loop): keep up to this many restart poses
                                  per ligand (<= 0 means 1, at most 16 and at most restarts) */
@@ -319,8 +321,8 @@ typedef struct {
   uint64_t align_poses;      /* alignment pose lanes evaluated (both alignments) */
   uint64_t torsion_angles;   /* torsion angle lanes of the scoring passes run */
   uint64_t angles_accepted;  /* of those, angles the bump check accepted (the ones Alg. 1 scores) */
-  uint64_t lookups;          /* pocket lookups evaluated */
-  uint64_t loads;            /* of those, lookups that issued a global load (inside the stored box) */
+  uint64_t lookups;          /* pocket lookups evaluated (the alignment's estimates are not lookups) */
+  uint64_t loads;            /* global loads issued: by lookups inside the stored box and by estimates */
   uint64_t sectors;          /* distinct 32-byte sectors those loads read, counted per warp-wide load */
   uint64_t pair_tests;       /* bump-check distance tests evaluated (angle lanes x pairs) */
   uint64_t lines;            /* distinct 128-byte lines those loads read, counted per warp-wide load */

@@ -1133,6 +1133,52 @@ void serve_loop(dock_ctx* ctx) {
 // C-ABI
 // ================================================================================================
 
+namespace {
+
+// Layout of a trilinear grid's screening cells: strides and number of cells; cells == 0 where none are
+// built (an axis past the fixed-point coordinates' range, or more than 2^28 cells, 2 GB).  The kernel's
+// index adds 0x45000 (the exponent bits of 2048.f) to each coordinate; the row is lengthened until that
+// bias plus any index stays below 2^32, so that one 64-bit multiply-add from a biased base address
+// finds a cell.
+size_t screen_layout(const dock_grid_desc& g, ScreenDev& sc, uint64_t& bias) {
+  const int most = 2000 - 2 * kScreenPad;
+  if (g.nx > most || g.ny > most || g.nz > most) return 0;
+  const uint64_t cz = g.nz - 1 + 2 * kScreenPad;
+  sc.cx = g.nx - 1 + 2 * kScreenPad;
+  sc.cy = g.ny - 1 + 2 * kScreenPad;
+  for (;; ++sc.cx) {
+    const uint64_t cells = (uint64_t)sc.cx * sc.cy * cz;
+    if (cells > (uint64_t)1 << 28) return 0;
+    bias = (0x45000ull * ((uint64_t)sc.cy * sc.cx + sc.cx + 1)) & 0xffffffffull;
+    if (bias + cells < (1ull << 32)) return cells;
+  }
+}
+
+// Quantisation of the field (launch_screen_range's result r): the smallest step with which every corner
+// of every cell fits 7 bits above its cell's base, a multiple of `mult` steps below 16.  False for a
+// field that is flat, or too large or small for the FP32 arithmetic around it.
+bool screen_steps(const float r[6], bool inside, ScreenDev& sc, float& inv_step) {
+  const double vmax = r[0], vmin = -(double)r[1], range = vmax - vmin, spread = r[2];
+  const double amax = std::max((double)r[0], (double)r[1]);
+  if (!(range > 1e-20 && amax < 1e20)) return false;
+  double best = 0;
+  for (int m = 1; m <= 100; ++m) {
+    const double step = std::max(spread / (125.0 - m), range / (125.0 + 15.0 * m));
+    if (best == 0 || step < best) best = step, sc.mult = (unsigned)m;
+  }
+  const float step = (float)(best * 1.0001);
+  inv_step = 1.0f / step;
+  sc.vmin = (float)vmin;
+  sc.units = kScreenUnits / step;
+  sc.quant = 0.5f + 1e-3f + (float)(amax / step) * 4e-7f;
+  sc.slope = (float)(((double)r[3] + r[4] + r[5]) / step) * 1.001f + 0.01f;
+  sc.vabs = (float)(amax / step) * 1.001f;
+  sc.inside = inside;
+  return true;
+}
+
+}  // namespace
+
 extern "C" {
 
 int dock_create(const dock_config* cfg, dock_ctx** out) {
@@ -1293,6 +1339,10 @@ int dock_load_pocket(dock_ctx* ctx, const dock_grid_desc* g, const float* host_v
   const bool empty = hi[0] < 0;
   if (empty)
     for (int a = 0; a < 3; ++a) lo[a] = 0, hi[a] = -1;
+  ScreenDev screen{};
+  uint64_t screen_bias = 0;
+  const size_t screen_cells = i16 || empty ? 0 : screen_layout(*g, screen, screen_bias);
+  const bool inside = lo[0] < 1 || lo[1] < 1 || lo[2] < 1 || hi[0] > g->nx - 2 || hi[1] > g->ny - 2 || hi[2] > g->nz - 2;
   cudaSetDevice(ctx->device);
   float* tmp = nullptr;
   Pocket P;
@@ -1314,10 +1364,38 @@ int dock_load_pocket(dock_ctx* ctx, const dock_grid_desc* g, const float* host_v
       e = cudaMemcpyAsync(P.cells, box.data(), box.size() * sizeof(int16_t), cudaMemcpyHostToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   } else {
-    e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), nv * sizeof(float), ctx->stream);
-    if (e == cudaSuccess) e = cudaMallocAsync(&P.cells, ncell * (g->dtype == DOCK_GRID_F16 ? 16 : 32), ctx->stream);
+    const bool f16 = g->dtype == DOCK_GRID_F16;
+    const size_t cell_bytes = (ncell * (f16 ? 16 : 32) + 255) & ~size_t(255);
+    // staging: the voxel values and the field's range
+    e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), (nv + 6) * sizeof(float), ctx->stream);
+    unsigned char* cells8 = nullptr;
+    if (e == cudaSuccess && screen_cells) {
+      // the screening cells live behind the pocket's own cells, in one allocation; where that does
+      // not fit the pocket is loaded without them
+      if (cudaMallocAsync(&P.cells, cell_bytes + 8 * screen_cells, ctx->stream) == cudaSuccess) {
+        cells8 = static_cast<unsigned char*>(P.cells) + cell_bytes;
+      } else {
+        cudaGetLastError();
+        P.cells = nullptr;
+      }
+    }
+    if (e == cudaSuccess && !P.cells) e = cudaMallocAsync(&P.cells, cell_bytes, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(tmp, host_values, nv * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
-    if (e == cudaSuccess) e = launch_pack_pocket(tmp, P.cells, g->nx, g->ny, g->nz, g->dtype == DOCK_GRID_F16, ctx->stream);
+    if (e == cudaSuccess) e = launch_pack_pocket(tmp, P.cells, g->nx, g->ny, g->nz, f16, ctx->stream);
+    if (e == cudaSuccess && cells8) {
+      float r[6];
+      e = cudaMemsetAsync(tmp + nv, 0, sizeof r, ctx->stream);
+      if (e == cudaSuccess)
+        e = launch_screen_range(tmp, g->nx, g->ny, g->nz, f16, !inside, reinterpret_cast<int*>(tmp + nv), ctx->stream);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(r, tmp + nv, sizeof r, cudaMemcpyDeviceToHost, ctx->stream);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+      float inv_step = 0.f;
+      if (e == cudaSuccess && screen_steps(r, inside, screen, inv_step)) {
+        e = launch_pack_screen(tmp, cells8, screen, g->nx, g->ny, g->nz, f16, inv_step, ctx->stream);
+        screen.base = reinterpret_cast<const void*>(reinterpret_cast<uintptr_t>(cells8) - 8 * (uintptr_t)screen_bias);
+        P.dev.screen = screen;
+      }
+    }
     if (tmp) cudaFreeAsync(tmp, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   }

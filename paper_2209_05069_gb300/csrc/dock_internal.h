@@ -20,6 +20,24 @@ inline int bucket_of(int n_atoms) { return (n_atoms - 1) / 32; }
 // (di, dj, dk) = (0,0,0), (1,0,0), (0,1,0), (1,1,0), (0,0,1), (1,0,1), (0,1,1), (1,1,1),
 // so one trilinear lookup is one 32-byte (FP32) or 16-byte (FP16) load.  One extra all-zero
 // cell at index (nx-1)(ny-1)(nz-1) serves every position outside the grid.
+struct ScreenDev {
+  const void* base;       // 8-byte cells at the address of the (biased) index the fixed-point coordinates
+                          // form; nullptr: every pose is scored in full
+  unsigned cx, cy;        // cells per row and per column, the padding of kScreenPad cells on each side included
+  float vmin;             // a cell's corner stands for vmin + step * (mult * base + corner)
+  float units;            // kScreenUnits / step: estimates are integers in units of step / kScreenUnits
+  unsigned mult;
+  float quant;            // error bound of one estimate in steps: voxel rounding
+  float slope;            // largest change per cell, summed over the axes, in steps
+  float vabs;             // largest |V| in steps
+  int inside;             // 1: a boundary voxel is nonzero (the field jumps to 0 at the grid's faces), so
+                          // only poses that stay inside the grid may be screened
+};
+constexpr int kScreenPad = 16;         // cells of padding around the grid: poses that reach past the grid are
+                                       // screened without clamping an index
+constexpr int kScreenFrac = 12;        // fraction bits of the fixed-point coordinates
+constexpr float kScreenUnits = 4096.f;
+
 struct PocketDev {
   const void* cells;
   int nx, ny, nz;
@@ -33,6 +51,8 @@ struct PocketDev {
   // holds voxels lo..hi of a box one voxel wider than the nonzero voxels on every side (its border
   // is zero; for an all-zero grid lo = -1, hi = 0), and a nearest-voxel index is clamped into it.
   float lox, loy, loz, hix, hiy, hiz;
+  // Screening cells of a trilinear grid (dock_screen.cuh).
+  ScreenDev screen;
 };
 
 // Packed ligands and result arrays of one batch, all in device memory.
@@ -106,6 +126,15 @@ struct LaunchCfg {
 // Builds the corner-packed cell array from voxel values (both in device memory).
 cudaError_t launch_pack_pocket(const float* values, void* cells, int nx, int ny, int nz, int f16,
                                cudaStream_t s);
+
+// Range of a trilinear grid's field: the extremes of its values, the largest difference between the
+// corners of one cell and the largest difference between neighbouring voxels along each axis.  `outside`:
+// the field continues as 0 outside the grid (else only the grid's own cells count).  Non-negative results
+// are stored as their bits: r = {max(vmax, 0), max(-vmin, 0), spread, dx, dy, dz}, zeroed by the caller.
+cudaError_t launch_screen_range(const float* values, int nx, int ny, int nz, int f16, int outside, int* r, cudaStream_t s);
+// Builds the screening cells (sc.cx x sc.cy x cz of them) from voxel values, both in device memory.
+cudaError_t launch_pack_screen(const float* values, void* cells, const ScreenDev& sc, int nx, int ny, int nz, int f16,
+                               float inv_step, cudaStream_t s);
 
 // Docks the work items (ligand << 10 | restart) of one atom bucket.  Every item of a ligand must
 // be in the same launch or in launches ordered on one stream (the last finished restart of a

@@ -25,24 +25,28 @@
 
 #include "dock_internal.h"
 
-// Register budget of the docking kernel.  dock_kernel: blocks of up to 256 threads, 4 of them
-// resident per SM (64 registers, a few spilled bytes outside the lookup loops).  Left to itself
-// ptxas takes 66-80 registers with 2-8 warps per item and over 100 with one; the bound measured
-// 7-15% faster with 2 or 4 warps per item and 19-43% faster with 8 on databases of 10^2-10^4
-// ligands.  dock_kernel_wide, the entry point of the FP32 grid with one warp per item: 96
-// registers (5 blocks of 128 threads per SM).  A sweep of one cap for every instantiation (64, 72,
-// 80, 96) on the uneven size mix and on 80-150-atom molecules kept 64 for the FP16 and int16 grids
-// and for 2 or more warps per item; FP32 with one warp per item and a pose tile of 2 ran 1-4% faster
-// per bucket at 96, the fastest shape of the 64-atom FP32 bucket.  A register cap (__maxnreg__) in
-// place of the launch bound generates other code: 64 registers that way made small serving batches
-// (8 warps per item) 8% slower at the median, so the bound stays.  DOCK_MAXNREG caps both entry
-// points at one count instead.
+// Register budgets of the docking kernel, by entry point.
+//  - dock_kernel: blocks of up to 256 threads, 4 of them resident per SM (64 registers, a few spilled
+//    bytes outside the lookup loops): 4 and 8 warps per item, and 2 on the integer grid.  Left to itself
+//    ptxas takes more, and the bound measured 7-15% faster with 2 or 4 warps per item and 19-43% faster
+//    with 8 on databases of 10^2-10^4 ligands.  A register cap (__maxnreg__) in place of the launch bound
+//    generates other code: 64 registers that way made small serving batches (8 warps per item) 8% slower
+//    at the median, so the bound stays.
+//  - dock_kernel_mid: 80 registers (3 blocks of 256 threads), 2 warps per item on a trilinear grid.  The
+//    screening loop wants them: 2,000 ligands of the uneven mix 9.5 ms (10.4 at 64, 11.4 at 96), 701 large
+//    molecules 14.6 ms (15.7 and 16.1).
+//  - dock_kernel_wide: 96 registers (5 blocks of 128 threads), one warp per item: 4,003 ligands 17.9 ms on
+//    FP32 cells (20.0 at 80, 33 at 64 with spills in the loops, 17.8 at 112), 18.6 on FP16 (21.7, 34.1),
+//    6,007 on the integer grid 15.8 (17.6, 36.5).
+// DOCK_MAXNREG caps all of them at one count instead.
 #ifdef DOCK_MAXNREG
 #define DOCK_KERNEL_BOUNDS __maxnreg__(DOCK_MAXNREG)
 #define DOCK_KERNEL_WIDE_BOUNDS __maxnreg__(DOCK_MAXNREG)
+#define DOCK_KERNEL_MID_BOUNDS __maxnreg__(DOCK_MAXNREG)
 #else
 #define DOCK_KERNEL_BOUNDS __launch_bounds__(256, 4)
 #define DOCK_KERNEL_WIDE_BOUNDS __maxnreg__(96)
+#define DOCK_KERNEL_MID_BOUNDS __maxnreg__(80)
 #endif
 
 // PTX load used for one FP32 corner-packed cell (32 bytes, one sector).
@@ -64,8 +68,9 @@ static_assert(kCnt <= 32, "one lane per counter flushes a warp's slot");
 __device__ __forceinline__ void cnt_add(int k, unsigned long long v) {
   if (v) atomicAdd(&g_cnt_smem[threadIdx.x >> 5][k], v);
 }
-// Lookup event of the active lanes: evaluated, loads issued, distinct sectors of those loads.
-__device__ __forceinline__ void cnt_lookup(bool issued, unsigned long long addr) {
+// Lookup event of the active lanes: evaluated (unless it is a screening estimate), loads issued,
+// distinct sectors of those loads.
+__device__ __forceinline__ void cnt_lookup(bool issued, unsigned long long addr, bool evaluated = true) {
   const unsigned act = __activemask();
   const int lane = threadIdx.x & 31;
   const unsigned issue = __ballot_sync(act, issued);
@@ -76,7 +81,7 @@ __device__ __forceinline__ void cnt_lookup(bool issued, unsigned long long addr)
   const unsigned ml = __match_any_sync(act, line);
   const unsigned line_leaders = __ballot_sync(act, issued && lane == __ffs(ml) - 1);
   if (lane == __ffs(act) - 1) {
-    cnt_add(kCntLookups, __popc(act));
+    if (evaluated) cnt_add(kCntLookups, __popc(act));
     cnt_add(kCntLoads, __popc(issue));
     cnt_add(kCntSectors, __popc(leaders));
     cnt_add(kCntLines, __popc(line_leaders));
@@ -392,6 +397,14 @@ __device__ __forceinline__ typename Acc<GT>::type lookup_at(const GridK& g, floa
   return lookup_acc<GT>(g, (x - g.ox) * g.inv_h, (y - g.oy) * g.inv_h, (z - g.oz) * g.inv_h);
 }
 
+constexpr int kDeal = 64;  // poses of an alignment dealt to a warp at a time (a pose tile of 1 or 2 divides it)
+
+}  // namespace dockgpu
+
+#include "dock_screen.cuh"
+
+namespace dockgpu {
+
 // ---- per-item shared memory ----------------------------------------------------------------------
 
 // Moving/fixed atom pairs from which the bump check of one bond is split over the item's warps.
@@ -564,19 +577,45 @@ __device__ __forceinline__ float3 centre_grid(const float4& cc, const GridK& g) 
 // Scores pose (i, j) for all N*N pairs (one pose per lane; the item's warps share the passes),
 // moves the ligand to the best one (ties: lowest i*N + j) and returns its flat index.  The
 // centroid is summed by warp 0 alone, so the result does not depend on the number of warps.
+//
+// Where poses can be screened they are dealt to the item's warps in blocks of kDeal, whether a warp
+// screens them or scores them all (each warp decides for itself).
+// With early exit and a trilinear grid that has screening cells, the poses are screened first
+// (dock_screen.cuh) and only those that can hold the best score are scored; the result is the same.
+// `scratch` is the warp's bump-pair buffer, unused during an alignment.
 template <int MAXN, int GT, int G, int T>
-__device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, const GridK& g, int wig, int lane,
-                           int grp) {
+__device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, const GridK& g, const PocketDev& pk,
+                           bool early_exit, float4* scratch, int wig, int lane, int grp) {
   if (wig == 0) align_centre(ws, n, lane);
   group_sync<G>(grp);
   const float4 cc = ws.bc;
   const float3 c = make_float3(cc.x, cc.y, cc.z);
   const float3 t = centre_grid(cc, g);
   const int NN = N * N;
+  constexpr int deal = GT != 2 && G < 8 ? kDeal : 32 * T;  // poses dealt to a warp at a time
   float best = -CUDART_INF_F;
   int bidx = 0x7fffffff;
-  for (int f0 = wig * 32 * T; f0 < NN; f0 += 32 * G * T)
-    align_pass<GT, T>(ws.u.rel, n, tab, N, g, t.x, t.y, t.z, f0, lane, best, bidx);
+  bool done = false;
+  // 8 warps per item are for small batches, where an item's latency counts: a warp has two or three passes
+  // then, and the dependent steps of screening cost more than its lookups save (12 ligands in the
+  // service 400 us screened, 330 not; 15 large molecules 777 and 673)
+  if constexpr (GT != 2 && G < 8) {
+    float mag;
+    if (early_exit && screen_usable(pk, ws.u.rel, n, t, g.inv_h, lane, mag)) {
+      // one warp per item: the torsion sweep's records behind the centred pose are free here
+      float* buf = G == 1 ? reinterpret_cast<float*>(ws.u.rel + MAXN) : reinterpret_cast<float*>(wig == 0 ? ws.pairs : scratch);
+      constexpr int cap = G == 1 ? 6 * MAXN : 4 * PairCap<MAXN>::value;
+      done = screen_align<GT, cap, G>(pk, g, ws.u.rel, n, tab, N, t, mag, wig, buf, lane, best, bidx);
+      DOCK_CNT(if (done && lane == 0) for (int f0 = wig * deal; f0 < NN; f0 += G * deal) for (int f = f0; f < min(f0 + deal, NN);
+               f += 32 * T) cnt_add(kCntAlignPoses, 32 * T);)
+    }
+  }
+  if (!done) {
+    best = -CUDART_INF_F, bidx = 0x7fffffff;
+    for (int f0 = wig * deal; f0 < NN; f0 += G * deal)
+      for (int f = f0; f < min(f0 + deal, NN); f += 32 * T)
+        align_pass<GT, T>(ws.u.rel, n, tab, N, g, t.x, t.y, t.z, f, lane, best, bidx);
+  }
   group_argmax<MAXN, G>(ws, best, bidx, wig, lane, grp);
   align_move(ws, n, tab, N, bidx, c, wig * 32 + lane, 32 * G);
   group_sync<G>(grp);
@@ -901,7 +940,7 @@ __device__ void dock_item(ItemSmem<MAXN>& ws, float4* xpairs, const float2* tab_
   if (wig == 0) start_pose(ws, n, bd.ids[l], p.seed, r, pk, lane);
   group_sync<G>(grp);
 
-  const int ai = align_phase<MAXN, GT, G, T>(ws, n, tab_al, p.N, g, wig, lane, grp);
+  const int ai = align_phase<MAXN, GT, G, T>(ws, n, tab_al, p.N, g, pk, p.early_exit != 0, xpairs, wig, lane, grp);
 
   for (int bi = 0; bi < B; ++bi) {
     const uint32_t ab = __ldg(bd.rot_ab + rb0 + bi);
@@ -916,7 +955,7 @@ __device__ void dock_item(ItemSmem<MAXN>& ws, float4* xpairs, const float2* tab_
     }
   }
 
-  const int pi = p.post_align ? align_phase<MAXN, GT, G, T>(ws, n, tab_al, p.N, g, wig, lane, grp) : -1;
+  const int pi = p.post_align ? align_phase<MAXN, GT, G, T>(ws, n, tab_al, p.N, g, pk, p.early_exit != 0, xpairs, wig, lane, grp) : -1;
   if (wig != 0) return;  // the rest is warp 0's
   const float s = pose_score<MAXN, GT>(ws, n, g, lane);
   const int cc = clash_count<MAXN>(ws, n, bd.excl + (size_t)a0 * kMaskWords, p.dc2, lane);
@@ -1056,12 +1095,15 @@ struct ResidentCache {
 
 DOCK_KERNEL_DEFINE(dock_kernel, DOCK_KERNEL_BOUNDS)
 DOCK_KERNEL_DEFINE(dock_kernel_wide, DOCK_KERNEL_WIDE_BOUNDS)
+DOCK_KERNEL_DEFINE(dock_kernel_mid, DOCK_KERNEL_MID_BOUNDS)
 
 // The entry point of an instantiation (only the one taken is instantiated).
 template <int MAXN, int GT, int G, int T>
 constexpr auto dock_kernel_entry() {
-  if constexpr (GT == 0 && G == 1)
+  if constexpr (G == 1)
     return &dock_kernel_wide<MAXN, GT, G, T>;
+  else if constexpr (GT != 2 && G == 2)
+    return &dock_kernel_mid<MAXN, GT, G, T>;
   else
     return &dock_kernel<MAXN, GT, G, T>;
 }
