@@ -96,3 +96,19 @@ def test_screening_at_the_largest_rotation_counts(dk, align):
     ref = _run(dk, pk, "f32", db, mk(0), (8, -1, 0, 2, 1))
     for shape in ((4, -1, 0, 1, 2), (8, -1, 0, 8, 1)):
         _same(ref, _run(dk, pk, "f32", db, mk(1), shape), (align, shape))
+
+
+@pytest.mark.parametrize("clash", [0.0, 0.5, 3.0, 9.0])
+def test_bump_check_against_the_oracle(dk, clash):
+    """The bump check over four angle passes at once, 100 angles (a last pass partly filled), at thresholds from
+    none to most of a molecule: decisions against the oracle, and the same rejected counts whether one or
+    eight warps share the check."""
+    from oracle import oracle
+    from tests import parity
+    pk, db = _field("workload"), _mixed(1)
+    prm = dk.Params.make(restarts=3, align_steps=8, torsion_steps=100, clash_dist=clash, seed=21)
+    res = _run(dk, pk, "f32", db, prm, (4, -1, 0, 1, 1))
+    _same(res, _run(dk, pk, "f32", db, prm, (8, -1, 0, 8, 1)), clash)
+    op = oracle.Params(restarts=3, align_steps=8, torsion_steps=100, clash_dist=clash, post_align=1, seed=21)
+    rep = parity.check(oracle, oracle.GridView.of(pk), db, res, op, threads=8)
+    assert not rep.failures, rep.failures[:5]
