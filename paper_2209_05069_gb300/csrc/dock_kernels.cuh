@@ -218,13 +218,16 @@ __device__ __forceinline__ GridK make_gridk(const PocketDev& p) {
 // integer grid is exact whatever the summation order.
 constexpr float kRound = 12582912.0f;  // 1.5 * 2^23: kRound + q has unit spacing for |q| < 2^22
 
-// Integer grid: the int16 value of the nearest voxel.  One round-down conversion per axis
-// (saturating) to a box-relative index, clamped by one unsigned min: an index past the box lands on
-// its far border, a negative one wraps to it, and the border is zero.
+// Integer grid: the int16 value of the nearest voxel.  Adding 2^23 with round-down leaves floor(u) in the
+// low mantissa bits (exact for 0 <= u < 2^23), and one fused add-and-min per axis turns the bits into a
+// box-relative index clamped to the far border: an index past the box lands there, and so does a
+// coordinate that is negative (its sum's bits fall below 2^23's and wrap), beyond 2^23 or not a number;
+// the border is zero.  The FMA pipe does the rounding, which as a conversion took the conversion pipe.
+__device__ __forceinline__ unsigned voxel_index(float u, int hi) {
+  return __viaddmin_u32(__float_as_uint(__fadd_rd(u, 8388608.f)), 0u - 0x4B000000u, (unsigned)hi);
+}
 __device__ __forceinline__ int voxel_value(const GridK& g, float u, float v, float w) {
-  const unsigned i = min((unsigned)__float2int_rd(u), (unsigned)g.ihix);
-  const unsigned j = min((unsigned)__float2int_rd(v), (unsigned)g.ihiy);
-  const unsigned k = min((unsigned)__float2int_rd(w), (unsigned)g.ihiz);
+  const unsigned i = voxel_index(u, g.ihix), j = voxel_index(v, g.ihiy), k = voxel_index(w, g.ihiz);
   const short* a = reinterpret_cast<const short*>(g.cells) + (k * (unsigned)g.ny1 + j) * (unsigned)g.nx1 + i;
   DOCK_CNT(cnt_lookup(true, (unsigned long long)a);)
   return __ldg(a);
