@@ -193,7 +193,10 @@ typedef struct {
 int dock_get_stats(dock_ctx* ctx, dock_stats* out);
 
 /* Launch shape of the docking kernel for one atom bucket (0: <=32 atoms, 1: <=64, 2: <=96,
- * 3: <=128, 4: <=160).  Results do not depend on the launch shape (tested bit for bit). */
+ * 3: <=128, 4: <=160).  Results do not depend on the launch shape (tested bit for bit).  Until a
+ * bucket's shape is set, each launch of a batch chooses one by the number of ligand-restarts it has to
+ * fill the GPU with and the bucket's atoms (8, 2 or 1 warps per ligand-restart, not persistent);
+ * dock_get_launch then reports the defaults named below. */
 typedef struct {
   int32_t warps_per_block;    /* 1..8 (default 8) */
   int32_t smem_carveout_pct;  /* preferred shared-memory share of the SM's L1/shared capacity,

@@ -671,6 +671,7 @@ struct dock_ctx {
   int fatal = 0;
   std::string fatal_msg;
   LaunchCfg launch_cfg[kNumBuckets];
+  int sms = 0;  // multiprocessors of the device
   int64_t latency_items = 0;  // serving batches of at most this many items use latency_launch
   int64_t latency_form_ligands = 0;  // serving batches of at most this many ligands: latency form
   uint64_t launch_version = 1;   // bumped by dock_set_launch (invalidates captured graphs)
@@ -691,9 +692,27 @@ struct dock_ctx {
 
 namespace {
 
-// Default launch shape of a bucket: 8 warps per block, driver carveout, persistent, two warps per
-// item, the shape the autotuner settles on for the uneven database and for most uniform batches.
-LaunchCfg default_launch(int bucket) { return LaunchCfg{8, -1, 1, bucket, 2, 1}; }
+// Default launch shape of a bucket: chosen by each launch (automatic_shape); reported as 8 warps per
+// block, driver carveout, persistent, two warps per item.
+LaunchCfg default_launch(int bucket) { return LaunchCfg{8, -1, 1, bucket, 2, 1, 1}; }
+
+// The shape of one bucket's launch: the one set for it, else by the ligand-restarts that fill the GPU
+// together with it (`items`) per SM.  Never persistent: plain grids let a bucket's blocks start where
+// the previous bucket's tail leaves SMs free (the uneven mix, 2,000 ligands: 9.2 ms plain, 10.1
+// persistent).  Measured in ms, 8 / 2 / 1 warps per item:
+//  - up to 8 per SM, 8 warps: 256 fragments 0.105 / 0.139 / 0.157, 1,200 items of the uneven mix on FP16
+//    0.359 / 0.403 / 0.563, of 15 large molecules 0.78 / 1.16 / 2.0; at 3,000 items 0.78 / 0.57 / 0.68;
+//  - from 30 per SM, one warp (20 are resident per SM; no barriers, the shared memory carveout halved for
+//    more L1): 6,000 items 1.53 / 1.03 / 0.95, 120,090 items 30.7 / 19.0 / 17.6 (18.2 with the driver's
+//    carveout); not above 64 atoms, where an item's shared memory leaves little L1 beside 20 of them:
+//    701 large molecules 21.6 / 14.6 / 15.6-23 (15.1 with one warp up to 96 atoms only);
+//  - between them two warps.
+LaunchCfg automatic_shape(const LaunchCfg& c, int bucket, int64_t items, int sms) {
+  if (!c.automatic) return c;
+  if (items <= (int64_t)8 * sms) return LaunchCfg{8, -1, 0, bucket, 8, 1, 0};
+  if (items >= (int64_t)30 * sms && bucket <= 1) return LaunchCfg{4, 50, 0, bucket, 1, 2, 0};
+  return LaunchCfg{8, -1, 0, bucket, 2, 1, 0};
+}
 
 // Records, on stream s, that work queued there reads pocket P (context lock held).  Events of
 // finished uses are recycled first, so the list holds only launches that may still be running.
@@ -741,11 +760,11 @@ void release_pocket(dock_ctx* ctx, Pocket& P) {
   P.cells = nullptr;
 }
 
+// The latency-oriented launch shape: one ligand-restart per block of 8 warps, all 8 on it.
+LaunchCfg latency_launch(int bucket) { return LaunchCfg{8, -1, 0, bucket, 8, 1, 0}; }
+
 // Launches every bucket of a prepared batch; the work is complete when stream s reaches the point
 // after the call.  Returns launches or a negative error.
-// The latency-oriented launch shape: one ligand-restart per block of 8 warps, all 8 on it.
-LaunchCfg latency_launch(int bucket) { return LaunchCfg{8, -1, 0, bucket, 8, 1}; }
-
 int launch_batch(dock_ctx* ctx, const PocketDev& pk, char* dev, const Layout& y, const Plan& plan,
                  const dock_params& prm, int form, cudaStream_t s, Fork* fork, std::string& err,
                  bool set_attributes = true, bool latency_shape = false) {
@@ -758,10 +777,16 @@ int launch_batch(dock_ctx* ctx, const PocketDev& pk, char* dev, const Layout& y,
     int order[kNumBuckets], nb = 0;
     for (int b = 0; b < kNumBuckets; ++b)
       if (plan.n_items[b]) order[nb++] = b;
-    std::sort(order, order + nb, [&](int p, int q) { return plan.bucket_cost[p] > plan.bucket_cost[q]; });
+    // the largest molecules first: their items run longest, so the last blocks are short ones (within a
+    // bucket items are sorted by cost)
+    std::reverse(order, order + nb);
     cudaError_t e = cudaSuccess;
     bool any_persistent = false;
-    auto shape = [&](int b) { return latency_shape ? latency_launch(b) : ctx->launch_cfg[b]; };
+    int64_t total = 0;
+    for (int i = 0; i < nb; ++i) total += plan.n_items[order[i]];
+    auto shape = [&](int b) {
+      return latency_shape ? latency_launch(b) : automatic_shape(ctx->launch_cfg[b], b, total, ctx->sms);
+    };
     for (int i = 0; i < nb; ++i) any_persistent |= shape(order[i]).persistent != 0;
     if (any_persistent) e = cudaMemsetAsync(bd.next_item, 0, 4 * kNumBuckets, s);
     if (nb > 1 && e == cudaSuccess) e = cudaEventRecord(fork->forked, s);
@@ -809,7 +834,7 @@ int launch_batch(dock_ctx* ctx, const PocketDev& pk, char* dev, const Layout& y,
   } else {
     for (int i = 0; i < plan.n_lig; ++i) {
       const int n = plan.lig_atom_off[i + 1] - plan.lig_atom_off[i];
-      LaunchCfg cfg = ctx->launch_cfg[bucket_of(n)];
+      LaunchCfg cfg = ctx->launch_cfg[bucket_of(n)];  // the default as reported
       cfg.persistent = 0;  // the plain form: one launch per ligand, one warp per restart
       const cudaError_t e = launch_dock_bucket(bucket_of(n), pk, bd, pd, items + plan.lig_item_off[i], prm.restarts,
                                                cfg, s);
@@ -860,10 +885,13 @@ int graph_launch(dock_ctx* ctx, int pocket_id, const PocketDev& pk, dock_batch* 
     ParamsDev pd = params_dev(b->params);
     pd.exec = ctx->exec;
     cudaError_t e = cudaSuccess;
+    int64_t total = 0;
+    for (int k = 0; k < kNumBuckets; ++k) total += b->plan.n_items[k];
     for (int k = 0; k < kNumBuckets && e == cudaSuccess; ++k)  // attributes outside the capture
       if (b->plan.n_items[k]) {
         e = form == DOCK_FORM_BATCHED
-                ? launch_dock_bucket(k, pk, bd, pd, nullptr, 0, ctx->launch_cfg[k], s, true)
+                ? launch_dock_bucket(k, pk, bd, pd, nullptr, 0, automatic_shape(ctx->launch_cfg[k], k, total, ctx->sms), s,
+                                     true)
                 : launch_latency_ligand(k, pk, bd, pd, -1, LatScratch{}, s, nullptr);
       }
     if (e != cudaSuccess) return err = fmt("kernel attributes: %s", cudaGetErrorString(e)), cuda_status(e);
@@ -1218,6 +1246,7 @@ int dock_create(const dock_config* cfg, dock_ctx** out) {
     dock_destroy(ctx.release());
     return DOCK_ERR_CUDA;
   }
+  ctx->sms = sms;
   ctx->latency_items = c.serve_latency_items < 0 ? 0 : c.serve_latency_items > 0 ? c.serve_latency_items : 2 * 4 * sms;
   ctx->latency_form_ligands = c.serve_latency_form < 0 ? 0 : c.serve_latency_form > 0 ? c.serve_latency_form : 1;
   if (!c.serve_off) ctx->server = std::thread(serve_loop, ctx.get());
@@ -1279,7 +1308,7 @@ int dock_set_launch(dock_ctx* ctx, int32_t bucket, const dock_launch_shape* sh) 
   const int tile = sh->pose_tile <= 0 ? 1 : sh->pose_tile;
   if (tile != 1 && (tile != 2 || g > 2))
     return ctx->fail(DOCK_ERR_INVALID, "pose_tile must be 1, or 2 with 1 or 2 warps per item");
-  ctx->launch_cfg[bucket] = LaunchCfg{sh->warps_per_block, sh->smem_carveout_pct, sh->persistent, bucket, g, tile};
+  ctx->launch_cfg[bucket] = LaunchCfg{sh->warps_per_block, sh->smem_carveout_pct, sh->persistent, bucket, g, tile, 0};
   ++ctx->launch_version;
   return DOCK_OK;
 }
@@ -1750,7 +1779,7 @@ int with_batch_view(dock_ctx* ctx, int pocket_id, const dock_batch* b, void* str
   v->params = params_dev(b->params);
   v->params.exec = ctx->exec;
   for (int k = 0; k < kNumBuckets; ++k) {
-    v->cfg[k] = ctx->launch_cfg[k];
+    v->cfg[k] = automatic_shape(ctx->launch_cfg[k], k, b->plan.n_items[k], ctx->sms);  // buckets one after another
     v->n_items[k] = b->plan.n_items[k];
     v->item_off[k] = b->plan.item_off[k];
   }

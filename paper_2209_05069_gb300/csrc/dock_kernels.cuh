@@ -1175,8 +1175,19 @@ cudaError_t launch_t(const PocketDev& pk, const BatchDev& b, const ParamsDev& p,
     blocks = blocks < resident * sms ? blocks : resident * sms;
     counter = b.next_item + cfg.counter_slot;
   }
-  kernel<<<blocks, wpb * 32, smem, s>>>(pk, b, p, items, n_items, wpb, counter);
-  return cudaGetLastError();
+  // the carveout goes with the launch, so that a captured launch keeps its own when another shape of the
+  // same kernel is launched later
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(blocks);
+  lc.blockDim = dim3(wpb * 32);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  at[0].val.sharedMemCarveout = cfg.smem_carveout >= 0 ? (unsigned)cfg.smem_carveout : (unsigned)cudaSharedmemCarveoutDefault;
+  lc.attrs = at;
+  lc.numAttrs = cfg.smem_carveout >= 0 ? 1 : 0;
+  return cudaLaunchKernelEx(&lc, kernel, pk, b, p, items, n_items, wpb, counter);
 }
 
 }  // namespace dockgpu

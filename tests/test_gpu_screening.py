@@ -1,4 +1,5 @@
-"""The alignment's screening (early_exit on a trilinear grid) changes no result.
+"""The alignment's screening (early_exit on a trilinear grid) and the launch shapes chosen by batch size
+change no result.
 
 Scoring every pose in full is the reference (early_exit=0; the oracle checks that path elsewhere): every
 output has to be equal bit for bit.  The fields and sizes are those where screening can go wrong: voxels at
@@ -96,6 +97,19 @@ def test_screening_at_the_largest_rotation_counts(dk, align):
     ref = _run(dk, pk, "f32", db, mk(0), (8, -1, 0, 2, 1))
     for shape in ((4, -1, 0, 1, 2), (8, -1, 0, 8, 1)):
         _same(ref, _run(dk, pk, "f32", db, mk(1), shape), (align, shape))
+
+
+@pytest.mark.parametrize("grid", ["f32", "i16"])
+@pytest.mark.parametrize("ligands", [1, 40, 41, 151, 152])
+def test_automatic_shapes_change_no_result(dk, ligands, grid):
+    """Batch sizes on both sides of the sizes at which a launch changes its shape (8 and 30 ligand-restarts
+    per SM: 1,216 and 4,560 on 152 SMs), in every atom bucket."""
+    pk = _field("workload")
+    if grid == "i16":
+        pk = pk.integer(1000)
+    db = synth.tile_db(_mixed(1), ligands)
+    prm = dk.Params.make(restarts=30, align_steps=8, torsion_steps=32, seed=9)
+    _same(_run(dk, pk, grid, db, prm, (4, -1, 0, 4, 1)), _run(dk, pk, grid, db, prm), (ligands, grid))
 
 
 @pytest.mark.parametrize("clash", [0.0, 0.5, 3.0, 9.0])
