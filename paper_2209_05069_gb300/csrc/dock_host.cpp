@@ -1106,13 +1106,18 @@ bool admit(dock_ctx* ctx, Slot& s, std::unique_lock<std::mutex>& lk) {
   return true;
 }
 
+// How long after its launch a serving batch is watched without sleeping between looks.
+constexpr int64_t kWatchNs = 400000;
+
 void serve_loop(dock_ctx* ctx) {
   cudaSetDevice(ctx->device);
   std::unique_lock<std::mutex> lk(ctx->mu);
   while (!ctx->stop) {
     bool progress = false, any_busy = false;
+    int64_t newest_launch = 0;
     for (Slot& s : ctx->slots) {
       if (!s.busy) continue;
+      newest_launch = std::max<int64_t>(newest_launch, s.t_launch);
       const cudaError_t q = cudaEventQuery(s.ev);
       if (q == cudaSuccess) {
         scatter_slot(ctx, s);
@@ -1146,8 +1151,14 @@ void serve_loop(dock_ctx* ctx) {
     if (ctx->fatal) ctx->done_cv.notify_all();
     if (progress) continue;
     if (any_busy) {
+      // A sleep of 20 us takes about 70 with the kernel's timer slack, most of a lone request's time on the
+      // GPU, so a batch is watched without sleeping while it is young enough to be such a one.
+      const bool young = now_ns() - newest_launch < kWatchNs;
       lk.unlock();
-      std::this_thread::sleep_for(std::chrono::microseconds(20));
+      if (young)
+        std::this_thread::yield();
+      else
+        std::this_thread::sleep_for(std::chrono::microseconds(20));
       lk.lock();
     } else {
       ctx->work_cv.wait_for(lk, std::chrono::milliseconds(50));
