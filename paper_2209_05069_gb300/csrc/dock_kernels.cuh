@@ -112,17 +112,16 @@ __device__ __forceinline__ int warp_sum_i(int v) {
   return v;
 }
 
-// Warp-wide (max score, lowest index among equal scores); every lane gets the result.
+// Warp-wide (max score, lowest index among equal scores); every lane gets the result.  Two integer
+// reductions and a shuffle in place of ten dependent shuffles: the argmax is on every bond's serial chain.
 __device__ __forceinline__ void warp_argmax(float& s, int& idx) {
-#pragma unroll
-  for (int o = 16; o; o >>= 1) {
-    const float s2 = __shfl_xor_sync(kFull, s, o);
-    const int i2 = __shfl_xor_sync(kFull, idx, o);
-    if (s2 > s || (s2 == s && i2 < idx)) {
-      s = s2;
-      idx = i2;
-    }
-  }
+  const int b = __float_as_int(s + 0.f);  // -0 counts as 0
+  const int key = b ^ ((b >> 31) & 0x7fffffff);  // orders as the scores do
+  const int m = __reduce_max_sync(kFull, key);
+  const int i = key == m ? idx : 0x7fffffff;
+  const int mi = __reduce_min_sync(kFull, i);
+  s = __shfl_sync(kFull, s, __ffs(__ballot_sync(kFull, key == m && idx == mi)) - 1);
+  idx = mi;
 }
 
 // SplitMix64 (Steele, Lea and Flood, OOPSLA 2014): output number k >= 1 of the generator
@@ -754,6 +753,7 @@ __device__ int torsion_phase(ItemSmem<MAXN>& ws, int n, int a, int b, const uint
     const int ways = split ? G : 1;
     float4* pairs = wig == 0 ? ws.pairs : xpairs;
     const int npairs = m * f;
+    const float inv_f = 1.0f / (float)f;  // pi / f: pi + 1/2 stays 1/320 clear of a multiple of f, far past the rounding
     unsigned clash_bits = 0;
     int cnt = 0;
     for (int p0 = wig * 32; p0 < npairs; p0 += 32 * ways) {
@@ -761,7 +761,7 @@ __device__ int torsion_phase(ItemSmem<MAXN>& ws, int n, int a, int b, const uint
       bool act = false;
       float C = 0.f, Pa = 0.f, Pb = 0.f;
       if (pi < npairs) {
-        const int km = pi / f, kf = pi - (pi / f) * f;
+        const int km = __float2int_rd(((float)pi + 0.5f) * inv_f), kf = pi - km * f;
         const int i = __float_as_int(ws.u.mov.B[km].w);
         const float4 q = ws.pos[i], xj = ws.pos[ws.fixed_idx[kf]];
         const float vx = q.x - pb.x, vy = q.y - pb.y, vz = q.z - pb.z;
@@ -793,11 +793,7 @@ __device__ int torsion_phase(ItemSmem<MAXN>& ws, int n, int a, int b, const uint
   group_sync<G>(grp);
   m = ws.bi[0];
   const unsigned clash_bits = ws.clash[lane];
-  {
-    int rej = 0;
-    for (int q = 0; q < nq; ++q) rej += __popc(__ballot_sync(kFull, (clash_bits >> q) & 1u));
-    rejected = rej;
-  }
+  rejected = __reduce_add_sync(kFull, __popc(clash_bits));
 
   // score every accepted angle: sum of lookups over the moving atoms (the rest is constant).  A group
   // is T passes of 32 angles (the angle tile): each lane scores angles (q0 + t) * 32 + lane, t < T,
