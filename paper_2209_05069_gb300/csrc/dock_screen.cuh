@@ -53,12 +53,17 @@ __device__ __forceinline__ bool screen_usable(const PocketDev& pk, const float4*
   return __all_sync(kFull, ok);
 }
 
-// The rotation of pose f = i * N + j with the grid scale folded in (align_pass's factors).
+// q / d by the reciprocal: (q + 1/2) / d stays 1/(2 d) clear of an integer, far past the rounding at q < 2^14,
+// d <= 160.
+__device__ __forceinline__ int quotient(int q, float inv_d) { return __float2int_rd(((float)q + 0.5f) * inv_d); }
+
+// The rotation of pose f = i * N + j with the grid scale folded in (align_pass's factors).  inv_N: 1 / N, or 0 for
+// an integer division.
 struct PoseRot {
   float r00, r01, r02, r11, r12, r20, r21, r22;
 };
-__device__ __forceinline__ PoseRot pose_rot(int f, const float2* tab, int N, float ih) {
-  const int i = f / N, j = f - (f / N) * N;
+__device__ __forceinline__ PoseRot pose_rot(int f, const float2* tab, int N, float inv_N, float ih) {
+  const int i = inv_N > 0.f ? quotient(f, inv_N) : f / N, j = f - i * N;
   const float2 ca = tab[i], cb = tab[j];  // (cos, sin)
   PoseRot r;
   r.r00 = cb.x * ih, r.r01 = cb.y * ca.y * ih, r.r02 = cb.y * ca.x * ih;
@@ -74,7 +79,7 @@ __device__ __forceinline__ float3 pose_at(const PoseRot& r, const float4& d, con
 // Estimates the poses f0 + lane + 32 t, t < T, in units of step / kScreenUnits, and puts them into the
 // lane's kScreenKeep best (top[0] the highest) and the best one left out (top[kScreenKeep]).  The low 9
 // bits of an entry hold the pass f / 32 (at most 511); 0 is no entry.
-template <int T, int U>
+template <int T, int U, bool kRecip>
 __device__ __forceinline__ void screen_pass(const PocketDev& pk, const float4* rel, int n, const float2* tab, int N,
                                             float ih, const float3& t3, int f0, int lane, unsigned (&top)[kScreenKeep + 1]) {
   const int NN = N * N;
@@ -84,7 +89,7 @@ __device__ __forceinline__ void screen_pass(const PocketDev& pk, const float4* r
 #pragma unroll
   for (int t = 0; t < T; ++t) {
     const int f = f0 + lane + 32 * t;
-    r[t] = pose_rot(f < NN ? f : 0, tab, N, ih);
+    r[t] = pose_rot(f < NN ? f : 0, tab, N, kRecip ? 1.0f / (float)N : 0.f, ih);
     acc[t] = 0;
     bases[t] = 0;
   }
@@ -130,7 +135,7 @@ __device__ __forceinline__ void screen_pass(const PocketDev& pk, const float4* r
 // Scores in full the pose f of every lane set in `mask` and folds them into (best, bidx), which end up
 // spread over the warp's lanes.  The (pose, atom) pairs are dealt to the lanes and each pose's values
 // are then summed in atom order by one lane: the additions of align_pass in their order.
-template <int GT, int CAP>
+template <int GT, int CAP, bool kRecip>
 __device__ __forceinline__ void screen_score(const GridK& g, const float4* rel, int n, const float2* tab, int N,
                                              const float3& t3, unsigned mask, int f, float* buf, int lane, float& best,
                                              int& bidx) {
@@ -141,11 +146,12 @@ __device__ __forceinline__ void screen_score(const GridK& g, const float4* rel, 
   __syncwarp();
   const int stride = n | 1;
   const int per = min((CAP - 16) / stride, 32);
+  const float inv_n = 1.0f / (float)n, inv_N = kRecip ? 1.0f / (float)N : 0.f;
   for (int c0 = 0; c0 < cnt; c0 += per) {
     const int m = min(per, cnt - c0);
     for (int q = lane; q < m * n; q += 32) {
-      const int c = q / n, a = q - c * n;
-      const float3 x = pose_at(pose_rot(list[c0 + c], tab, N, g.inv_h), rel[a], t3);
+      const int c = kRecip ? quotient(q, inv_n) : q / n, a = q - c * n;
+      const float3 x = pose_at(pose_rot(list[c0 + c], tab, N, inv_N, g.inv_h), rel[a], t3);
       val[c * stride + a] = lookup<GT>(g, x.x, x.y, x.z);
     }
     __syncwarp();
@@ -175,6 +181,9 @@ __device__ bool screen_align(const PocketDev& pk, const GridK& g, const float4* 
   // registers: 9.5, against 11.4 for 2 x 2 at 96).  Prefetching the next atom's cells instead was
   // no faster (9.3 against 8.7 on the FP16 grid).
   constexpr int T = G == 1 ? 2 : 1, U = G == 1 ? 2 : 4;
+  // Reciprocals for the pose and pair indices with one warp per item (4,003 uneven ligands 17.3 -> 16.6 ms);
+  // at the 80 registers of 2 warps per item they spill (18.2 -> 18.8) and the divisions stay.
+  constexpr bool kRecip = G == 1;
   const int NN = N * N;
   if (wig * kDeal >= NN) return true;  // no pose of this warp
   const float fn = (float)n;
@@ -189,9 +198,9 @@ __device__ bool screen_align(const PocketDev& pk, const GridK& g, const float4* 
   for (int f0 = wig * kDeal; f0 < NN; f0 += G * kDeal) {
     int f = f0;
     for (; f < f0 + kDeal && NN - f > 32 * (T - 1) + 8; f += 32 * T)
-      screen_pass<T, U>(pk, rel, n, tab, N, g.inv_h, start, f, lane, top);
+      screen_pass<T, U, kRecip>(pk, rel, n, tab, N, g.inv_h, start, f, lane, top);
     if (T > 1 && f < f0 + kDeal && NN - f > 8) {  // half a pass
-      screen_pass<1, U>(pk, rel, n, tab, N, g.inv_h, start, f, lane, top);
+      screen_pass<1, U, kRecip>(pk, rel, n, tab, N, g.inv_h, start, f, lane, top);
       f += 32;
     }
     if (f < min(f0 + kDeal, NN)) tail = f;
@@ -219,7 +228,7 @@ __device__ bool screen_align(const PocketDev& pk, const GridK& g, const float4* 
       if (k != 0) break;
       continue;
     }
-    screen_score<GT, CAP>(g, rel, n, tab, N, t3, mask, k == -2 ? tail + lane : (int)(e & 511u) * 32 + lane, buf, lane, b, bi);
+    screen_score<GT, CAP, kRecip>(g, rel, n, tab, N, t3, mask, k == -2 ? tail + lane : (int)(e & 511u) * 32 + lane, buf, lane, b, bi);
     if (k == -1) {
       // the line: the score just found in units of the estimates, less the bound
       float s0 = b;
