@@ -870,7 +870,7 @@ def main():
                    "l2": "flushed before each timed step (256 MiB write)", "parallelism": f"ligand shards x{world}",
                    "launch": {b: [t["warps_per_block"], t["smem_carveout"], t["persistent"], t["warps_per_item"],
                                   t.get("pose_tile", 1)] for b, t in tuning.items()}
-                   if tuning else "default (8 warps/block, driver carveout, persistent, 2 warps per item, tile 1)",
+                   if tuning else "default (chosen per launch by the batch's ligand-restarts per SM and the bucket)",
                    "launch_fields": "warps per block, carveout %, persistent, warps per item, pose tile"},
         "clocks": clk, "e2e": e2e, "gpu_launches": launches, "roofline": roofline, "cpu_baseline": cpu,
         "per_ligand_form": per_lig, "latency": serving,

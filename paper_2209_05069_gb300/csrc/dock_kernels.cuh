@@ -10,7 +10,8 @@
 // Mapping onto the warp (the paper's batched design gives one warp one ligand, lanes over atoms;
 // here lanes own poses so every lane stays busy whatever the ligand size):
 //  * alignment: lane = one of the N*N rotations; the lane rotates every atom (broadcast from
-//    shared memory) and sums its lookups; a warp argmax picks the pose.
+//    shared memory) and sums its lookups; a warp argmax picks the pose.  On a trilinear grid with early
+//    exit the poses are estimated first and only those that can win are summed (dock_screen.cuh).
 //  * torsion sweep: lane = one torsion angle.  The moving atoms' positions are written as
 //    x(theta) = c + cos(theta) r + sin(theta) w (c on the axis, r and w perpendicular), so one
 //    angle costs 6 FMA per atom before its lookup.  For the bump check every moving/fixed pair
@@ -1033,9 +1034,9 @@ __host__ __device__ constexpr size_t table_bytes(int N, int A) {
 // takes item b*(wpb/G) + q; otherwise (persistent form) every group pulls items from the counter
 // until the list is exhausted.
 //
-// One kernel body, two entry points with their own register budgets.  The body is a macro so that
+// One kernel body, three entry points with their own register budgets.  The body is a macro so that
 // each entry point is compiled as this kernel written out in full: moving it into a device function
-// called by both, even an inlined one, changed the code generated for the 8-warps-per-item kernel of
+// called by them, even an inlined one, changed the code generated for the 8-warps-per-item kernel of
 // small serving batches (ptxas reserved all 16 named barriers for it instead of 2, and their median
 // latency rose 8%).
 #define DOCK_KERNEL_DEFINE(NAME, BOUNDS)                                                                                     \
