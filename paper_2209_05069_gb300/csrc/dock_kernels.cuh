@@ -28,7 +28,8 @@
 
 // Register budgets of the docking kernel, by entry point.
 //  - dock_kernel: blocks of up to 256 threads, 4 of them resident per SM (64 registers, a few spilled
-//    bytes outside the lookup loops): 4 and 8 warps per item, and 2 on the integer grid.  Left to itself
+//    bytes outside the lookup loops): 4 and 8 warps per item, and on the integer grid 2, or one with a
+//    pose tile of 1 (which the tuner takes for 10,000 ligands there: 451k ligands/s, 403k at 96).  Left to itself
 //    ptxas takes more, and the bound measured 7-15% faster with 2 or 4 warps per item and 19-43% faster
 //    with 8 on databases of 10^2-10^4 ligands.  A register cap (__maxnreg__) in place of the launch bound
 //    generates other code: 64 registers that way made small serving batches (8 warps per item) 8% slower
@@ -1112,7 +1113,7 @@ DOCK_KERNEL_DEFINE(dock_kernel_mid, DOCK_KERNEL_MID_BOUNDS)
 // The entry point of an instantiation (only the one taken is instantiated).
 template <int MAXN, int GT, int G, int T>
 constexpr auto dock_kernel_entry() {
-  if constexpr (G == 1)
+  if constexpr (G == 1 && !(GT == 2 && T == 1))
     return &dock_kernel_wide<MAXN, GT, G, T>;
   else if constexpr (GT != 2 && G == 2)
     return &dock_kernel_mid<MAXN, GT, G, T>;
