@@ -7,7 +7,7 @@
 // pose index kept are those of scoring every pose; no estimate enters a result.
 //
 // What it saves: an FP32 lookup gathers a 32-byte cell and is bound by the L1 data pipe (about 23
-// wavefronts per warp-wide load, 13-18 for the 16-byte FP16 cells).  A screening cell is 8 bytes (about 9
+// wavefronts per warp-wide load, 13-18 for the 16-byte FP16 cells).  A screening cell is 8 bytes (about 12
 // wavefronts, and twice to four times the cells per byte of L1), and the coordinates are fixed point, so
 // the index and the fractions are bit fields and the interpolation is exact integer arithmetic.  The same
 // idea with 16-byte cells of FP16 polynomial coefficients was 1.2 times slower: bound by the data pipe.
