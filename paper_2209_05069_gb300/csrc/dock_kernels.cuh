@@ -621,6 +621,7 @@ __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, 
         align_pass<GT, T>(ws.u.rel, n, tab, N, g, t.x, t.y, t.z, f, lane, best, bidx);
   }
   group_argmax<MAXN, G>(ws, best, bidx, wig, lane, grp);
+  bidx = bidx < NN ? bidx : 0;  // no pose scored above -infinity (a field past FP16's or FP32's range): pose 0
   align_move(ws, n, tab, N, bidx, c, wig * 32 + lane, 32 * G);
   group_sync<G>(grp);
   return bidx;
@@ -1016,6 +1017,7 @@ __device__ void finish_restart(const ItemSmem<MAXN>& ws, const BatchDev& bd, con
     }
   }
   warp_argmax(best, br);
+  br = br < p.R ? br : 0;  // no score above -infinity: restart 0
   const float* src = bd.rs_xyz + ((size_t)a0 * p.R + (size_t)br * n) * 3;
   for (int i = lane; i < 3 * n; i += 32) bd.out_xyz[(size_t)a0 * 3 + i] = __ldcg(src + i);
   if (lane == 0) {

@@ -75,7 +75,7 @@ __device__ __forceinline__ int lat_pick(const float2* cand, int passes, int lane
     }
   }
   warp_argmax(best, idx);
-  return idx;
+  return idx == 0x7fffffff ? 0 : idx;  // no pose scored above -infinity: pose 0, as in align_phase
 }
 
 // Counter build: adds the warp's counts to the launch's totals (nothing in the normal build).
