@@ -237,6 +237,13 @@ def executed_work(dock, local, pk, grid_dtype, db, prm, bucket, tuning):
     return c
 
 
+def launch_fields(table):
+    """A tuning table's shapes for the record; "automatic" where each launch chooses its own."""
+    return {str(b): "automatic" if t.get("automatic") else
+            [t["warps_per_block"], t["smem_carveout"], t["persistent"], t["warps_per_item"], t.get("pose_tile", 1)]
+            for b, t in (table or {}).items()}
+
+
 def _bucket_and_grid(kernel):
     """(MAXN, grid type) of a docking-kernel name such as dock_kernel<64, 0, 2, 1>."""
     return tuple(x.strip() for x in kernel.split("<", 1)[1].split(",")[:2])
@@ -447,15 +454,13 @@ def run_plateau(args):
         served = size / (time.perf_counter() - t0)
         rows.append({"ligands": size, "batched": batched, "served_e2e": served, "per_ligand": per_lig,
                      "batched_over_per_ligand": batched / per_lig,
-                     "launch": {k: [v["warps_per_block"], v["smem_carveout"], v["persistent"], v["warps_per_item"],
-                                    v.get("pose_tile", 1)] for k, v in (tuning or {}).items()}})
+                     "launch": launch_fields(tuning)})
         print(json.dumps(rows[-1]), flush=True)
     ctx.close()
     print(json.dumps({"mode": "plateau", "workload": w.name, "grid": f"{w.grid}^3 @ {w.spacing} A",
                       "grid_dtype": grid_dtype, "restarts": w.restarts, "torsion_steps": w.torsion_steps,
                       "unit": UNIT, "rows": rows,
-                      "launch": {k: [v["warps_per_block"], v["smem_carveout"], v["persistent"], v["warps_per_item"],
-                                     v.get("pose_tile", 1)] for k, v in (tuning or {}).items()}}),
+                      "launch": launch_fields(tuning)}),
           flush=True)
     return 0
 
@@ -493,8 +498,7 @@ def run_classes(args):
             prm = dock.Params.make(restarts=w.restarts, align_steps=w.align_steps, torsion_steps=w.torsion_steps,
                                    clash_dist=w.clash_dist, seed=2209)
             tuned = autotune.tune(ctx, pid, db, prm, reps=1)
-            row["launch"] = {str(b): [t["warps_per_block"], t["smem_carveout"], t["persistent"], t["warps_per_item"],
-                                      t.get("pose_tile", 1)] for b, t in tuned.items()}
+            row["launch"] = launch_fields(tuned)
         modes = (1, 0) if args.early_exit == "both" else (int(args.early_exit),)
         forms = ((dock.DOCK_FORM_BATCHED, "batched", db), (dock.DOCK_FORM_PER_LIGAND, "per_ligand", db.slice(0, 64)))
         for ee in modes:
@@ -728,7 +732,7 @@ def main():
         per_lig = {"value": sub.n_lig / (ms / 1e3), "unit": UNIT, "sample": f"first {sub.n_lig} ligands",
                    "launches": sub.n_lig}
         # one ligand at a time with 8 warps per ligand-restart (the latency-oriented shape)
-        saved = [ctx.get_launch(k) for k in range(5)]
+        saved = [ctx.resolve_launch(k, 0) for k in range(5)]
         for k in range(5):
             ctx.set_launch(k, 8, -1, 0, 8)
         ctx.batch_launch(pid, b2, dock.DOCK_FORM_PER_LIGAND, sptr)
@@ -739,6 +743,9 @@ def main():
         torch.cuda.synchronize()
         ms8 = e0.elapsed_time(e1)
         for k, sh in enumerate(saved):
+            if sh["automatic"]:
+                ctx.reset_launch(k)
+                continue
             ctx.set_launch(k, sh["warps_per_block"], sh["smem_carveout_pct"], sh["persistent"], sh["warps_per_item"],
                            sh["pose_tile"])
         per_lig["ms_per_ligand"] = ms / sub.n_lig
@@ -803,7 +810,7 @@ def main():
     alu = flops / mean_s / 1e12
     bytes_per_lookup = {"f16": 16, "i16": 2}.get(grid_dtype, 32)
     gt = {"f16": 1, "i16": 2}.get(grid_dtype, 0)
-    sh = ctx.get_launch(dom["bucket"])
+    sh = ctx.resolve_launch(dom["bucket"], dom["ligands"] * w.restarts)
     entry = "dock_kernel_wide" if gt == 0 and sh["warps_per_item"] == 1 else "dock_kernel"
     kernel = f"{entry}<{32 * (dom['bucket'] + 1)}, {gt}, {sh['warps_per_item']}, {sh['pose_tile']}>"
     launch_s = dom["ms_per_launch"] / 1e3
@@ -868,9 +875,8 @@ def main():
                    "torsion_steps": w.torsion_steps, "grid": f"{w.grid}^3 @ {w.spacing} A", "grid_dtype": grid_dtype,
                    "select_poses": {"k": prm.k, "rmsd": prm.select_rmsd},
                    "l2": "flushed before each timed step (256 MiB write)", "parallelism": f"ligand shards x{world}",
-                   "launch": {b: [t["warps_per_block"], t["smem_carveout"], t["persistent"], t["warps_per_item"],
-                                  t.get("pose_tile", 1)] for b, t in tuning.items()}
-                   if tuning else "default (chosen per launch by the batch's ligand-restarts per SM and the bucket)",
+                   "launch": launch_fields(tuning) if tuning else
+                   "default (chosen per launch by the batch's ligand-restarts per SM and the bucket)",
                    "launch_fields": "warps per block, carveout %, persistent, warps per item, pose tile"},
         "clocks": clk, "e2e": e2e, "gpu_launches": launches, "roofline": roofline, "cpu_baseline": cpu,
         "per_ligand_form": per_lig, "latency": serving,

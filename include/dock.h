@@ -220,6 +220,12 @@ int dock_set_launch(dock_ctx* ctx, int32_t bucket, const dock_launch_shape* shap
 /* Reads the launch shape of one bucket.  Error: DOCK_ERR_INVALID. */
 int dock_get_launch(dock_ctx* ctx, int32_t bucket, dock_launch_shape* shape);
 
+/* Reads the shape that the bucket's launch runs with in a dock_batch_launch of `items` ligand-restarts (over all
+ * buckets).  Returns 1 if that launch chooses the shape itself (none is set), 0 if it is the one set.  A program
+ * that sets shapes for a while restores a bucket that was 1 with dock_set_launch(ctx, bucket, NULL); setting what
+ * dock_get_launch reports would fix its shape.  Error: DOCK_ERR_INVALID. */
+int dock_resolve_launch(dock_ctx* ctx, int32_t bucket, int64_t items, dock_launch_shape* shape);
+
 /* ---- pocket -------------------------------------------------------------------------------- */
 
 /* Uploads a pocket grid (Section 4.1: the pocket is shared read-only by all ligands) and builds

@@ -42,9 +42,10 @@ def tune(ctx: "dock.Context", pocket_id: int, db, params: "dock.Params", warps=W
 
     Shapes whose warps per item do not divide warps per block, or with a tile of 2 and more than 2
     warps per item, are skipped.  With ``joint`` the per-bucket winners are then checked against a
-    few shapes common to all buckets with the buckets running side by side (see _joint).  Returns
-    {bucket: {"warps_per_block", "smem_carveout", "persistent", "warps_per_item", "pose_tile", "ms",
-    "ligands", "tried"[, "joint"]}}.
+    few shapes common to all buckets and the shapes each launch chooses itself, with the buckets running
+    side by side (see _joint).  Returns {bucket: {"warps_per_block", "smem_carveout", "persistent",
+    "warps_per_item", "pose_tile", "ms", "ligands", "tried"[, "automatic", "joint"]}}; with "automatic" true
+    no shape is set for the bucket and the shape fields are what ``get_launch`` reports for it.
     """
     n = np.diff(db.atom_off)
     table = {}
@@ -80,7 +81,7 @@ def tune(ctx: "dock.Context", pocket_id: int, db, params: "dock.Params", warps=W
                     "pose_tile": tl, "ms": ms, "ligands": int(idx.size),
                     "tried": [[w, c, q, g_, t_, round(t, 4)] for w, c, q, g_, t_, t in tried]}
         samples.append(idx)
-    if joint and len(table) > 1:
+    if joint and table:
         _joint(ctx, pocket_id, db, params, table, np.concatenate(samples), reps, log)
     return table
 
@@ -88,20 +89,19 @@ def tune(ctx: "dock.Context", pocket_id: int, db, params: "dock.Params", warps=W
 def _joint(ctx, pocket_id, db, params, table, idx, reps, log):
     """The buckets of a batch run side by side, so each bucket's fastest shape alone need not be
     the fastest set.  Times the per-bucket winners against the few shapes that did best summed over
-    all buckets, each applied to every bucket, and against the library defaults, on the buckets'
-    samples docked together; keeps the fastest set."""
+    all buckets, each applied to every bucket, and against the library default (no shape set: each launch
+    chooses its own), on the buckets' samples docked together; keeps the fastest set."""
     tried = {b: {tuple(t[:5]): t[5] for t in row["tried"]} for b, row in table.items()}
     common = set.intersection(*(set(d) for d in tried.values()))
     ranked = sorted(common, key=lambda sh: sum(tried[b][sh] for b in tried))[:3]
     sets = [("per bucket", {b: _shape(r) for b, r in table.items()})]
     sets += [(f"all {sh}", {b: sh for b in table}) for sh in ranked]
-    sets.append(("library default", _defaults(ctx, table)))
+    sets.append(("library default", {b: None for b in table}))
     batch = ctx.batch_create(db.subset(idx), params)
     results = []
     try:
         for name, shapes in sets:
-            for b, sh in shapes.items():
-                ctx.set_launch(b, *sh)
+            _use(ctx, shapes)
             ctx.batch_launch(pocket_id, batch)
             ctx.batch_wait(batch)
             best = float("inf")
@@ -116,31 +116,38 @@ def _joint(ctx, pocket_id, db, params, table, idx, reps, log):
     finally:
         ctx.batch_destroy(batch)
     best, name, shapes = min(results, key=lambda t: t[0])
+    _use(ctx, shapes)
     for b, sh in shapes.items():
-        ctx.set_launch(b, *sh)
         row = table[b]
-        _set_shape(row, sh)
+        _set_shape(ctx, b, row, sh)
         row["joint"] = {"chosen": name, "ms": round(best, 4), "tried": [[n_, round(t, 4)] for t, n_, _ in results]}
 
 
 def _shape(row):
-    """(warps per block, carveout, persistent, warps per item, pose tile) of a table row."""
-    return (row["warps_per_block"], row["smem_carveout"], row["persistent"], row["warps_per_item"],
-            row.get("pose_tile", 1))
+    """(warps per block, carveout, persistent, warps per item, pose tile) of a table row; None: no shape set."""
+    if row.get("automatic"):
+        return None
+    return (int(row["warps_per_block"]), int(row["smem_carveout"]), int(row.get("persistent", 0)),
+            int(row.get("warps_per_item", 1)), int(row.get("pose_tile", 1)))
 
 
-def _set_shape(row, sh):
+def _set_shape(ctx, bucket, row, sh):
+    """Records shape ``sh`` of a bucket (None: what get_launch reports while none is set)."""
+    row["automatic"] = sh is None
+    if sh is None:
+        g = ctx.get_launch(bucket)
+        sh = (g["warps_per_block"], g["smem_carveout_pct"], g["persistent"], g["warps_per_item"], g["pose_tile"])
     row["warps_per_block"], row["smem_carveout"], row["persistent"], row["warps_per_item"], row["pose_tile"] = sh
 
 
-def _defaults(ctx, buckets):
-    """The library's default launch shape of each bucket (what dock_set_launch with NULL restores)."""
-    out = {}
-    for b in buckets:
-        ctx.reset_launch(b)
-        g = ctx.get_launch(b)
-        out[b] = (g["warps_per_block"], g["smem_carveout_pct"], g["persistent"], g["warps_per_item"], g["pose_tile"])
-    return out
+def _use(ctx, shapes):
+    """Sets each bucket's shape; None leaves the choice to each launch (dock_set_launch with NULL), which is not
+    the shape that get_launch then reports."""
+    for b, sh in shapes.items():
+        if sh is None:
+            ctx.reset_launch(int(b))
+        else:
+            ctx.set_launch(int(b), *sh)
 
 
 def _time_batch(ctx, pocket_id, batch, reps):
@@ -157,27 +164,28 @@ def _time_batch(ctx, pocket_id, batch, reps):
 
 def confirm(ctx: "dock.Context", pocket_id: int, db, params: "dock.Params", table: dict, reps: int = 3,
             log=None) -> dict:
-    """Docks the whole of ``db`` with the tuned table and with the library defaults and keeps the
+    """Docks the whole of ``db`` with the tuned table and with the library default (no shape set) and keeps the
     faster (the tuner times samples of at most a few thousand ligands per bucket, whose balance
     can differ from the whole database's).  Records both times in every row under "confirm"."""
     if not table:
         return table
     tuned = {b: _shape(r) for b, r in table.items()}
+    defaults = {b: None for b in table}
     batch = ctx.batch_create(db, params)
     try:
-        apply(ctx, table)
+        _use(ctx, tuned)
         t_tuned = _time_batch(ctx, pocket_id, batch, reps)
-        defaults = _defaults(ctx, table)
+        _use(ctx, defaults)
         t_default = _time_batch(ctx, pocket_id, batch, reps)
     finally:
         ctx.batch_destroy(batch)
     shapes, chosen = (tuned, "tuned") if t_tuned <= t_default else (defaults, "library default")
     if log:
         log(f"whole database: tuned {t_tuned:.3f} ms, library default {t_default:.3f} ms -> {chosen}")
+    _use(ctx, shapes)
     for b, sh in shapes.items():
-        ctx.set_launch(b, *sh)
         row = table[b]
-        _set_shape(row, sh)
+        _set_shape(ctx, b, row, sh)
         row["confirm"] = {"chosen": chosen, "tuned_ms": round(t_tuned, 4), "default_ms": round(t_default, 4),
                           "ligands": int(db.n_lig)}
     return table
@@ -185,9 +193,7 @@ def confirm(ctx: "dock.Context", pocket_id: int, db, params: "dock.Params", tabl
 
 def apply(ctx: "dock.Context", table: dict):
     """Applies a table produced by :func:`tune` (e.g. loaded from JSON)."""
-    for b, row in table.items():
-        ctx.set_launch(int(b), int(row["warps_per_block"]), int(row["smem_carveout"]), int(row.get("persistent", 0)),
-                       int(row.get("warps_per_item", 1)), int(row.get("pose_tile", 1)))
+    _use(ctx, {b: _shape(row) for b, row in table.items()})
 
 
 def save(table: dict, path: str, **meta):

@@ -1333,6 +1333,16 @@ int dock_get_launch(dock_ctx* ctx, int32_t bucket, dock_launch_shape* sh) {
   return DOCK_OK;
 }
 
+int dock_resolve_launch(dock_ctx* ctx, int32_t bucket, int64_t items, dock_launch_shape* sh) {
+  if (!ctx) return DOCK_ERR_INVALID;
+  std::lock_guard<std::mutex> lk(ctx->mu);
+  if (bucket < 0 || bucket >= kNumBuckets || items < 0 || !sh)
+    return ctx->fail(DOCK_ERR_INVALID, "bad bucket, negative items or NULL shape");
+  const LaunchCfg c = automatic_shape(ctx->launch_cfg[bucket], bucket, items, ctx->sms);
+  *sh = dock_launch_shape{c.warps_per_block, c.smem_carveout, c.persistent, c.warps_per_item, c.tile};
+  return ctx->launch_cfg[bucket].automatic ? 1 : 0;
+}
+
 int dock_get_stats(dock_ctx* ctx, dock_stats* out) {
   if (!ctx || !out) return DOCK_ERR_INVALID;
   std::lock_guard<std::mutex> lk(ctx->mu);

@@ -37,7 +37,7 @@ SYMBOLS = ["dock_create", "dock_destroy", "dock_last_error", "dock_load_pocket",
            "dock_validate_ligands", "dock_get_stats",
            "dock_submit_ligands", "dock_poll", "dock_results", "dock_batch_create", "dock_batch_launch",
            "dock_batch_results", "dock_batch_destroy", "dock_batch_work", "dock_batch_launch_noalloc", "dock_set_launch", "dock_batch_wait",
-           "dock_get_launch", "dock_gather_peak", "dock_exec_counters"]
+           "dock_get_launch", "dock_resolve_launch", "dock_gather_peak", "dock_exec_counters"]
 
 NOALLOC_SCRATCH_BYTES = 16 << 20
 DEVICE_RESULT_FIELDS = ["score", "best_restart", "xyz", "clash_count", "restart_score", "restart_clash", "align_idx",
@@ -168,6 +168,7 @@ def lib(counters: bool = False):
             L.dock_batch_wait.argtypes = [vp, vp]
             L.dock_set_launch.argtypes = [vp, C.c_int32, _P(LaunchShape)]
             L.dock_get_launch.argtypes = [vp, C.c_int32, _P(LaunchShape)]
+            L.dock_resolve_launch.argtypes = [vp, C.c_int32, C.c_int64, _P(LaunchShape)]
             L.dock_batch_launch_noalloc.argtypes = [vp, C.c_int32, vp, _P(DeviceResults), vp]
             L.dock_gather_peak.argtypes = [vp, C.c_int32, _P(C.c_double)]
             L.dock_validate_ligands.argtypes = [_P(LigandBatch), _P(Params), C.c_char_p, C.c_size_t]
@@ -303,6 +304,13 @@ class Context:
         sh = LaunchShape()
         self._check(self._lib.dock_get_launch(self.h, bucket, C.byref(sh)))
         return {k: int(getattr(sh, k)) for k, _ in LaunchShape._fields_}
+
+    def resolve_launch(self, bucket: int, items: int) -> dict:
+        """The shape one bucket's launch runs with in a batch of ``items`` ligand-restarts; "automatic": the launch
+        chooses it (no shape is set for the bucket)."""
+        sh = LaunchShape()
+        auto = self._check(self._lib.dock_resolve_launch(self.h, bucket, items, C.byref(sh)))
+        return dict({k: int(getattr(sh, k)) for k, _ in LaunchShape._fields_}, automatic=bool(auto))
 
     def stats(self) -> dict:
         st = Stats()
