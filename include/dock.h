@@ -65,9 +65,10 @@ typedef struct {
                                  DOCK_ERR_TIMEOUT for unfinished tickets (default 120000) */
   int32_t serve_latency_items; /* serving batches of at most this many ligand-restarts run with the
                                  latency-oriented launch shape (8 warps per ligand-restart, one per
-                                 block, not persistent), larger ones with the dock_set_launch shapes:
-                                 a small batch then finishes sooner, a large one keeps the
-                                 throughput shape.  0: twice the items 8-warp blocks fill the GPU
+                                 block, not persistent), larger ones with the dock_set_launch shapes
+                                 (with none set: 1 or 2 warps per ligand-restart, see
+                                 dock_launch_shape): a small batch then finishes sooner, a large one
+                                 keeps the throughput shape.  0: twice the items 8-warp blocks fill the GPU
                                  with at once (4 blocks per SM); -1: never */
   int32_t serve_latency_form; /* serving batches of at most this many ligands are docked in the
                                  latency form (DOCK_FORM_LATENCY: one ligand at a time over the whole
@@ -195,7 +196,8 @@ int dock_get_stats(dock_ctx* ctx, dock_stats* out);
 /* Launch shape of the docking kernel for one atom bucket (0: <=32 atoms, 1: <=64, 2: <=96,
  * 3: <=128, 4: <=160).  Results do not depend on the launch shape (tested bit for bit).  Until a
  * bucket's shape is set, each launch of a batch chooses one by the number of ligand-restarts it has to
- * fill the GPU with and the bucket's atoms (8, 2 or 1 warps per ligand-restart, not persistent);
+ * fill the GPU with and the bucket's atoms (8, 2 or 1 warps per ligand-restart, not persistent; in the
+ * serving loop dock_config::serve_latency_items decides on 8);
  * dock_get_launch then reports the defaults named below. */
 typedef struct {
   int32_t warps_per_block;    /* 1..8 (default 8) */

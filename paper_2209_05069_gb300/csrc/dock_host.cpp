@@ -707,9 +707,11 @@ LaunchCfg default_launch(int bucket) { return LaunchCfg{8, -1, 1, bucket, 2, 1, 
 //    carveout); not above 64 atoms, where an item's shared memory leaves little L1 beside 20 of them:
 //    701 large molecules 21.6 / 14.6 / 15.6-23 (15.1 with one warp up to 96 atoms only);
 //  - between them two warps.
-LaunchCfg automatic_shape(const LaunchCfg& c, int bucket, int64_t items, int sms) {
+// `eight`: whether 8 warps may be chosen.  Not in a serving launch, where dock_config::serve_latency_items alone
+// says which batches take them.
+LaunchCfg automatic_shape(const LaunchCfg& c, int bucket, int64_t items, int sms, bool eight = true) {
   if (!c.automatic) return c;
-  if (items <= (int64_t)8 * sms) return LaunchCfg{8, -1, 0, bucket, 8, 1, 0};
+  if (eight && items <= (int64_t)8 * sms) return LaunchCfg{8, -1, 0, bucket, 8, 1, 0};
   if (items >= (int64_t)30 * sms && bucket <= 1) return LaunchCfg{4, 50, 0, bucket, 1, 2, 0};
   return LaunchCfg{8, -1, 0, bucket, 2, 1, 0};
 }
@@ -767,7 +769,7 @@ LaunchCfg latency_launch(int bucket) { return LaunchCfg{8, -1, 0, bucket, 8, 1, 
 // after the call.  Returns launches or a negative error.
 int launch_batch(dock_ctx* ctx, const PocketDev& pk, char* dev, const Layout& y, const Plan& plan,
                  const dock_params& prm, int form, cudaStream_t s, Fork* fork, std::string& err,
-                 bool set_attributes = true, bool latency_shape = false) {
+                 bool set_attributes = true, bool latency_shape = false, bool serving = false) {
   const BatchDev bd = batch_pointers(dev, y, plan.n_lig);
   ParamsDev pd = params_dev(prm);
   pd.exec = ctx->exec;
@@ -785,7 +787,7 @@ int launch_batch(dock_ctx* ctx, const PocketDev& pk, char* dev, const Layout& y,
     int64_t total = 0;
     for (int i = 0; i < nb; ++i) total += plan.n_items[order[i]];
     auto shape = [&](int b) {
-      return latency_shape ? latency_launch(b) : automatic_shape(ctx->launch_cfg[b], b, total, ctx->sms);
+      return latency_shape ? latency_launch(b) : automatic_shape(ctx->launch_cfg[b], b, total, ctx->sms, !serving);
     };
     for (int i = 0; i < nb; ++i) any_persistent |= shape(order[i]).persistent != 0;
     if (any_persistent) e = cudaMemsetAsync(bd.next_item, 0, 4 * kNumBuckets, s);
@@ -1074,7 +1076,7 @@ bool admit(dock_ctx* ctx, Slot& s, std::unique_lock<std::mutex>& lk) {
       const bool lat_form = (int64_t)L <= ctx->latency_form_ligands;
       const bool latency = (int64_t)L * R <= ctx->latency_items;
       rc = launch_batch(ctx, pit->second.dev, s.dev, s.y, s.plan, prm, lat_form ? DOCK_FORM_LATENCY : DOCK_FORM_BATCHED,
-                        s.stream, &s.fork, err, true, latency);
+                        s.stream, &s.fork, err, true, latency, true);
       if (rc >= 0) note_use(ctx, pit->second, s.stream);
       if (rc >= 0 && lat_form) ctx->stats.latency_form_batches += 1;
       else if (rc >= 0 && latency) ctx->stats.latency_batches += 1;
