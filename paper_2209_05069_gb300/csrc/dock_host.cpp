@@ -31,6 +31,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include <sys/prctl.h>
 #include <unistd.h>
 
 #include <cuda_runtime.h>
@@ -620,6 +621,7 @@ struct Slot {
   char* host = nullptr;
   size_t host_cap = 0;
   bool busy = false;
+  bool small = false;  // in the latency form or shape
   int64_t t_launch = 0;
   Layout y{};
   Plan plan;
@@ -667,6 +669,7 @@ struct dock_ctx {
   int64_t queued = 0;            // ligands submitted but not yet admitted
   std::vector<Slot> slots;
   std::thread server;
+  std::atomic<bool> wake{false};  // set with mu held by calls that the serving loop has to see at once
   bool stop = false;
   int fatal = 0;
   std::string fatal_msg;
@@ -1078,6 +1081,7 @@ bool admit(dock_ctx* ctx, Slot& s, std::unique_lock<std::mutex>& lk) {
       rc = launch_batch(ctx, pit->second.dev, s.dev, s.y, s.plan, prm, lat_form ? DOCK_FORM_LATENCY : DOCK_FORM_BATCHED,
                         s.stream, &s.fork, err, true, latency, true);
       if (rc >= 0) note_use(ctx, pit->second, s.stream);
+      s.small = lat_form || latency;
       if (rc >= 0 && lat_form) ctx->stats.latency_form_batches += 1;
       else if (rc >= 0 && latency) ctx->stats.latency_batches += 1;
       if (rc >= 0)
@@ -1108,18 +1112,32 @@ bool admit(dock_ctx* ctx, Slot& s, std::unique_lock<std::mutex>& lk) {
   return true;
 }
 
-// How long after its launch a serving batch is watched without sleeping between looks.
+// How long after its launch a small serving batch is watched without sleeping between looks.
 constexpr int64_t kWatchNs = 400000;
+
+// Looks at the running batches' events until one has finished, a call wakes the loop or the time is `until`.  Called
+// without the context lock: submit, poll and results come and go meanwhile (with the lock taken for each look, a
+// mutex that is not fair kept other threads out of it for up to the whole window).
+void watch(dock_ctx* ctx, const std::vector<cudaEvent_t>& running, int64_t until) {
+  while (!ctx->wake.load(std::memory_order_acquire) && now_ns() < until) {
+    for (cudaEvent_t e : running)
+      if (cudaEventQuery(e) != cudaErrorNotReady) return;
+    std::this_thread::yield();
+  }
+}
 
 void serve_loop(dock_ctx* ctx) {
   cudaSetDevice(ctx->device);
+  prctl(PR_SET_TIMERSLACK, 1000UL);  // this thread's sleeps: 1 us late at most in place of 50
+  std::vector<cudaEvent_t> running;
   std::unique_lock<std::mutex> lk(ctx->mu);
   while (!ctx->stop) {
+    ctx->wake.store(false, std::memory_order_relaxed);
     bool progress = false, any_busy = false;
-    int64_t newest_launch = 0;
+    int64_t watch_until = 0;
+    running.clear();
     for (Slot& s : ctx->slots) {
       if (!s.busy) continue;
-      newest_launch = std::max<int64_t>(newest_launch, s.t_launch);
       const cudaError_t q = cudaEventQuery(s.ev);
       if (q == cudaSuccess) {
         scatter_slot(ctx, s);
@@ -1132,6 +1150,8 @@ void serve_loop(dock_ctx* ctx) {
         progress = true;
       } else {
         any_busy = true;
+        running.push_back(s.ev);
+        if (s.small) watch_until = std::max<int64_t>(watch_until, s.t_launch + kWatchNs);
         // watchdog: a batch that runs past the stall limit stops admission; its work is left to
         // finish (a kernel cannot be cancelled) and unfinished tickets report DOCK_ERR_TIMEOUT
         const int64_t ran_ms = (now_ns() - s.t_launch) / 1000000;
@@ -1153,12 +1173,11 @@ void serve_loop(dock_ctx* ctx) {
     if (ctx->fatal) ctx->done_cv.notify_all();
     if (progress) continue;
     if (any_busy) {
-      // A sleep of 20 us takes about 70 with the kernel's timer slack, most of a lone request's time on the
-      // GPU, so a batch is watched without sleeping while it is young enough to be such a one.
-      const bool young = now_ns() - newest_launch < kWatchNs;
+      // A sleep is a good part of a lone request's time on the GPU, so a small batch is watched without one while
+      // it is young enough to be such a request; larger ones run for milliseconds and are looked at every 20 us.
       lk.unlock();
-      if (young)
-        std::this_thread::yield();
+      if (now_ns() < watch_until)
+        watch(ctx, running, watch_until);
       else
         std::this_thread::sleep_for(std::chrono::microseconds(20));
       lk.lock();
@@ -1272,6 +1291,7 @@ int dock_destroy(dock_ctx* ctx) {
   {
     std::lock_guard<std::mutex> g(ctx->mu);
     ctx->stop = true;
+    ctx->wake.store(true, std::memory_order_release);
   }
   ctx->work_cv.notify_all();
   if (ctx->server.joinable()) ctx->server.join();
@@ -1576,6 +1596,7 @@ int dock_submit_ligands(dock_ctx* ctx, int32_t pocket_id, const dock_ligand_batc
   if (L > 0) ctx->pending.push_back(id);
   ctx->tickets[id] = std::move(T);
   *ticket = id;
+  ctx->wake.store(true, std::memory_order_release);
   ctx->work_cv.notify_all();
   return DOCK_OK;
 }
