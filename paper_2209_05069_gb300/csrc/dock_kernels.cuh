@@ -598,7 +598,7 @@ __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, 
   const int NN = N * N;
   constexpr int deal = GT != 2 && G < 8 ? kDeal : 32 * T;  // poses dealt to a warp at a time
   float best = -CUDART_INF_F;
-  int bidx = 0x7fffffff;
+  int bidx = 0;  // kept where no pose scores above -infinity (a field past FP16's or FP32's range)
   bool done = false;
   // 8 warps per item are for small batches, where an item's latency counts: a warp has two or three passes
   // then, and the dependent steps of screening cost more than its lookups save (12 ligands in the
@@ -615,13 +615,12 @@ __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, 
     }
   }
   if (!done) {
-    best = -CUDART_INF_F, bidx = 0x7fffffff;
+    best = -CUDART_INF_F, bidx = 0;
     for (int f0 = wig * deal; f0 < NN; f0 += G * deal)
       for (int f = f0; f < min(f0 + deal, NN); f += 32 * T)
         align_pass<GT, T>(ws.u.rel, n, tab, N, g, t.x, t.y, t.z, f, lane, best, bidx);
   }
   group_argmax<MAXN, G>(ws, best, bidx, wig, lane, grp);
-  bidx = bidx < NN ? bidx : 0;  // no pose scored above -infinity (a field past FP16's or FP32's range): pose 0
   align_move(ws, n, tab, N, bidx, c, wig * 32 + lane, 32 * G);
   group_sync<G>(grp);
   return bidx;
@@ -1008,7 +1007,7 @@ __device__ void finish_restart(const ItemSmem<MAXN>& ws, const BatchDev& bd, con
   __syncwarp();
   __threadfence();
   float best = -CUDART_INF_F;
-  int br = 0x7fffffff;
+  int br = 0;  // kept where no score is above -infinity
   for (int q = lane; q < p.R; q += 32) {
     const float v = __ldcg(bd.restart_score + (size_t)l * p.R + q);
     if (v > best) {
@@ -1017,7 +1016,6 @@ __device__ void finish_restart(const ItemSmem<MAXN>& ws, const BatchDev& bd, con
     }
   }
   warp_argmax(best, br);
-  br = br < p.R ? br : 0;  // no score above -infinity: restart 0
   const float* src = bd.rs_xyz + ((size_t)a0 * p.R + (size_t)br * n) * 3;
   for (int i = lane; i < 3 * n; i += 32) bd.out_xyz[(size_t)a0 * 3 + i] = __ldcg(src + i);
   if (lane == 0) {

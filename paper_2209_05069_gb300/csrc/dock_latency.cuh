@@ -65,7 +65,7 @@ __device__ __forceinline__ void lat_align_pass(const float4* rel, int n, const f
 // warp gets it.
 __device__ __forceinline__ int lat_pick(const float2* cand, int passes, int lane) {
   float best = -CUDART_INF_F;
-  int idx = 0x7fffffff;
+  int idx = 0;  // kept where no pose scores above -infinity, as in align_phase
   for (int q = lane; q < passes; q += 32) {
     const float2 c = __ldcg(cand + q);
     const int i = __float_as_int(c.y);
@@ -75,7 +75,7 @@ __device__ __forceinline__ int lat_pick(const float2* cand, int passes, int lane
     }
   }
   warp_argmax(best, idx);
-  return idx == 0x7fffffff ? 0 : idx;  // no pose scored above -infinity: pose 0, as in align_phase
+  return idx;
 }
 
 // Counter build: adds the warp's counts to the launch's totals (nothing in the normal build).
@@ -126,7 +126,7 @@ __device__ __forceinline__ bool lat_passes_then_last(ItemSmem<MAXN>& ws, const f
   if (q < passes) {
     const float3 t = centre_grid(ws.bc, g);
     float best = -CUDART_INF_F;
-    int bidx = 0x7fffffff;
+    int bidx = 0;
     lat_align_pass<GT, kLatUnroll>(ws.u.rel, n, tab, p.N, g, t.x, t.y, t.z, q * 32, lane, best, bidx);
     warp_argmax(best, bidx);
     if (lane == 0) sc.cand[(size_t)r * passes + q] = make_float2(best, __int_as_float(bidx));

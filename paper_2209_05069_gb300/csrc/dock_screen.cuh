@@ -213,7 +213,7 @@ __device__ bool screen_align(const PocketDev& pk, const GridK& g, const float4* 
   const unsigned m = __reduce_max_sync(kFull, top[0]);  // 0: every pose of the warp is in the tail
   const int who = __ffs(__ballot_sync(kFull, top[0] == m)) - 1;
   float b = -CUDART_INF_F;
-  int bi = 0x7fffffff;
+  int bi = 0;
   unsigned line = 0;
   bool ok = true;
 #pragma unroll 1
