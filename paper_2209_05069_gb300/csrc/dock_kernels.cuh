@@ -582,10 +582,11 @@ __device__ __forceinline__ float3 centre_grid(const float4& cc, const GridK& g) 
 // moves the ligand to the best one (ties: lowest i*N + j) and returns its flat index.  The
 // centroid is summed by warp 0 alone, so the result does not depend on the number of warps.
 //
-// Where poses can be screened they are dealt to the item's warps in blocks of kDeal, whether a warp
-// screens them or scores them all (each warp decides for itself).
 // With early exit and a trilinear grid that has screening cells, the poses are screened first
-// (dock_screen.cuh) and only those that can hold the best score are scored; the result is the same.
+// (dock_screen.cuh) and only those that can hold the best score are scored; the result is the same.  They are
+// then dealt to the item's warps in blocks of kDeal, whether a warp screens them or scores them all (each warp
+// decides for itself), and by single passes otherwise: in blocks of kDeal, 25-64 poses on 4 warps ran 19-23%
+// slower, on 2 warps 13-16%.
 // `scratch` is the warp's bump-pair buffer, unused during an alignment.
 template <int MAXN, int GT, int G, int T>
 __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, const GridK& g, const PocketDev& pk,
@@ -596,9 +597,9 @@ __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, 
   const float3 c = make_float3(cc.x, cc.y, cc.z);
   const float3 t = centre_grid(cc, g);
   const int NN = N * N;
-  constexpr int deal = GT != 2 && G < 8 ? kDeal : 32 * T;  // poses dealt to a warp at a time
   float best = -CUDART_INF_F;
   int bidx = 0;  // kept where no pose scores above -infinity (a field past FP16's or FP32's range)
+  int deal = 32 * T;  // poses dealt to a warp at a time
   bool done = false;
   // 8 warps per item are for small batches, where an item's latency counts: a warp has two or three passes
   // then, and the dependent steps of screening cost more than its lookups save (12 ligands in the
@@ -606,6 +607,7 @@ __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, 
   if constexpr (GT != 2 && G < 8) {
     float mag;
     if (early_exit && screen_usable(pk, ws.u.rel, n, t, g.inv_h, lane, mag)) {
+      deal = kDeal;
       // one warp per item: the torsion sweep's records behind the centred pose are free here
       float* buf = G == 1 ? reinterpret_cast<float*>(ws.u.rel + MAXN) : reinterpret_cast<float*>(wig == 0 ? ws.pairs : scratch);
       constexpr int cap = G == 1 ? 6 * MAXN : 4 * PairCap<MAXN>::value;
