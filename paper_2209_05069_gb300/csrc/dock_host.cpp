@@ -697,7 +697,7 @@ namespace {
 
 // Default launch shape of a bucket: chosen by each launch (automatic_shape); reported as 8 warps per
 // block, driver carveout, persistent, two warps per item.
-LaunchCfg default_launch(int bucket) { return LaunchCfg{8, -1, 1, bucket, 2, 1, 1}; }
+LaunchCfg default_launch(int bucket) { return LaunchCfg{8, -1, 1, bucket, 2, 1, 0, 1}; }
 
 // The shape of one bucket's launch: the one set for it, else by the ligand-restarts that fill the GPU
 // together with it (`items`) per SM.  Never persistent: plain grids let a bucket's blocks start where
@@ -714,9 +714,9 @@ LaunchCfg default_launch(int bucket) { return LaunchCfg{8, -1, 1, bucket, 2, 1, 
 // says which batches take them.
 LaunchCfg automatic_shape(const LaunchCfg& c, int bucket, int64_t items, int sms, bool eight = true) {
   if (!c.automatic) return c;
-  if (eight && items <= (int64_t)8 * sms) return LaunchCfg{8, -1, 0, bucket, 8, 1, 0};
-  if (items >= (int64_t)30 * sms && bucket <= 1) return LaunchCfg{4, 50, 0, bucket, 1, 2, 0};
-  return LaunchCfg{8, -1, 0, bucket, 2, 1, 0};
+  if (eight && items <= (int64_t)8 * sms) return LaunchCfg{8, -1, 0, bucket, 8, 1, 0, 0};
+  if (items >= (int64_t)30 * sms && bucket <= 1) return LaunchCfg{4, 50, 0, bucket, 1, 2, 0, 0};
+  return LaunchCfg{8, -1, 0, bucket, 2, 1, 0, 0};
 }
 
 // Records, on stream s, that work queued there reads pocket P (context lock held).  Events of
@@ -766,7 +766,7 @@ void release_pocket(dock_ctx* ctx, Pocket& P) {
 }
 
 // The latency-oriented launch shape: one ligand-restart per block of 8 warps, all 8 on it.
-LaunchCfg latency_launch(int bucket) { return LaunchCfg{8, -1, 0, bucket, 8, 1, 0}; }
+LaunchCfg latency_launch(int bucket) { return LaunchCfg{8, -1, 0, bucket, 8, 1, 0, 0}; }
 
 // Launches every bucket of a prepared batch; the work is complete when stream s reaches the point
 // after the call.  Returns launches or a negative error.
@@ -801,6 +801,7 @@ int launch_batch(dock_ctx* ctx, const PocketDev& pk, char* dev, const Layout& y,
       if (i > 0) e = cudaStreamWaitEvent(t, fork->forked, 0);
       LaunchCfg cfg = shape(b);
       cfg.counter_slot = b;
+      cfg.together = (int)std::min<int64_t>(total, INT32_MAX);
       if (e == cudaSuccess)
         e = launch_dock_bucket(b, pk, bd, pd, items + plan.item_off[b], plan.n_items[b], cfg, t, set_attributes);
       if (e == cudaSuccess && i > 0) e = cudaEventRecord(fork->joined[b], t);
@@ -1341,7 +1342,7 @@ int dock_set_launch(dock_ctx* ctx, int32_t bucket, const dock_launch_shape* sh) 
   const int tile = sh->pose_tile <= 0 ? 1 : sh->pose_tile;
   if (tile != 1 && (tile != 2 || g > 2))
     return ctx->fail(DOCK_ERR_INVALID, "pose_tile must be 1, or 2 with 1 or 2 warps per item");
-  ctx->launch_cfg[bucket] = LaunchCfg{sh->warps_per_block, sh->smem_carveout_pct, sh->persistent, bucket, g, tile, 0};
+  ctx->launch_cfg[bucket] = LaunchCfg{sh->warps_per_block, sh->smem_carveout_pct, sh->persistent, bucket, g, tile, 0, 0};
   ++ctx->launch_version;
   return DOCK_OK;
 }

@@ -121,6 +121,7 @@ struct LaunchCfg {
   int warps_per_item;    // warps docking one (ligand, restart): 1, 2, 4 or 8
   int tile;              // poses (alignment) or angles (torsion) one lane scores per pass: 1, or 2
                          // with 1 or 2 warps per item
+  int together;          // ligand-restarts that fill the GPU together with this launch (0: its own)
   int automatic;         // 1: the bucket's default, whose shape each launch chooses (automatic_shape); the other
                          // fields are then what dock_get_launch reports
 };

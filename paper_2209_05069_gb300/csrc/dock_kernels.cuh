@@ -582,7 +582,7 @@ __device__ __forceinline__ float3 centre_grid(const float4& cc, const GridK& g) 
 // moves the ligand to the best one (ties: lowest i*N + j) and returns its flat index.  The
 // centroid is summed by warp 0 alone, so the result does not depend on the number of warps.
 //
-// With early exit and a trilinear grid that has screening cells, the poses are screened first
+// With early exit and a trilinear grid that has screening cells, the poses are screened first where that pays
 // (dock_screen.cuh) and only those that can hold the best score are scored; the result is the same.  They are
 // then dealt to the item's warps in blocks of kDeal, whether a warp screens them or scores them all (each warp
 // decides for itself), and by single passes otherwise: in blocks of kDeal, 25-64 poses on 4 warps ran 19-23%
@@ -601,10 +601,7 @@ __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, 
   int bidx = 0;  // kept where no pose scores above -infinity (a field past FP16's or FP32's range)
   int deal = 32 * T;  // poses dealt to a warp at a time
   bool done = false;
-  // 8 warps per item are for small batches, where an item's latency counts: a warp has two or three passes
-  // then, and the dependent steps of screening cost more than its lookups save (12 ligands in the
-  // service 400 us screened, 330 not; 15 large molecules 777 and 673)
-  if constexpr (GT != 2 && G < 8) {
+  if constexpr (screen_compiled(MAXN, GT, G)) {
     float mag;
     if (early_exit && screen_usable(pk, ws.u.rel, n, t, g.inv_h, lane, mag)) {
       deal = kDeal;
@@ -638,8 +635,11 @@ __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, 
 // One pass at a time (two chains each) left the check bound by its own latency: with 4 at once, one large
 // molecule in the latency form went from 221 to 197 us, 12 requests in the service from 375 to 325 us, 2,000
 // ligands on the integer grid from 5.13 to 5.00 ms; 2 at once: 214 us, 328 us and 5.2 ms.
-constexpr int kBumpTile = 4;
+// FP16 cells with 4 warps per item take 2 at a time, with which its 64 registers spill 48 bytes of loads (176 with 4): one
+// large molecule per launch 1.25 times slower with 4 than with 2.
+__host__ __device__ constexpr int bump_tile(int gt, int g) { return gt == 1 && g == 4 ? 2 : 4; }
 
+template <int kBumpTile>
 __device__ __forceinline__ unsigned check_pairs(const float4* pairs, int cnt, const float2* tab, int A, int nq,
                                                 float dc2, bool early_exit, unsigned prior, int lane) {
   __syncwarp();
@@ -782,13 +782,13 @@ __device__ int torsion_phase(ItemSmem<MAXN>& ws, int n, int a, int b, const uint
       const unsigned bal = __ballot_sync(kFull, act);
       const int na = __popc(bal);
       if (cnt + na > CAP) {
-        clash_bits |= check_pairs(pairs, cnt, tab, A, nq, dc2, early_exit, clash_bits, lane);
+        clash_bits |= check_pairs<bump_tile(GT, G)>(pairs, cnt, tab, A, nq, dc2, early_exit, clash_bits, lane);
         cnt = 0;
       }
       if (act) pairs[cnt + __popc(bal & lt)] = make_float4(C, Pa, Pb, 0.f);
       cnt += na;
     }
-    clash_bits |= check_pairs(pairs, cnt, tab, A, nq, dc2, early_exit, clash_bits, lane);
+    clash_bits |= check_pairs<bump_tile(GT, G)>(pairs, cnt, tab, A, nq, dc2, early_exit, clash_bits, lane);
     if (!split)
       ws.clash[lane] = clash_bits;
     else if (clash_bits)
@@ -1165,13 +1165,14 @@ cudaError_t launch_t(const PocketDev& pk, const BatchDev& b, const ParamsDev& p,
     }
   }
   if (n_items <= 0) return cudaSuccess;
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int per_block = wpb / G;
   int blocks = (n_items + per_block - 1) / per_block;
   unsigned* counter = nullptr;
   if (cfg.persistent && b.next_item) {
-    int resident = 0, sms = 0;
+    int resident = 0;
     if (!lookup_resident(&resident) || resident < 1) resident = 1;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     blocks = blocks < resident * sms ? blocks : resident * sms;
     counter = b.next_item + cfg.counter_slot;
   }
@@ -1187,7 +1188,10 @@ cudaError_t launch_t(const PocketDev& pk, const BatchDev& b, const ParamsDev& p,
   at[0].val.sharedMemCarveout = cfg.smem_carveout >= 0 ? (unsigned)cfg.smem_carveout : (unsigned)cudaSharedmemCarveoutDefault;
   lc.attrs = at;
   lc.numAttrs = cfg.smem_carveout >= 0 ? 1 : 0;
-  return cudaLaunchKernelEx(&lc, kernel, pk, b, p, items, n_items, wpb, counter);
+  PocketDev pocket = pk;
+  const int together = cfg.together > n_items ? cfg.together : n_items;
+  if (!screening_pays(MAXN, GT, G, p.N, together, sms)) pocket.screen.base = nullptr;
+  return cudaLaunchKernelEx(&lc, kernel, pocket, b, p, items, n_items, wpb, counter);
 }
 
 }  // namespace dockgpu

@@ -24,6 +24,29 @@
 
 namespace dockgpu {
 
+// Kernels that hold the screening code.  Not with 8 warps per item: that is for small batches, where an item's
+// latency counts; a warp has two or three passes then, and the dependent steps of screening cost more than its
+// lookups save (12 ligands in the service 400 us screened, 330 not; 15 large molecules 777 and 673).  On FP16 cells a
+// lookup costs half an FP32 one and screening gains less: nothing with 4 warps per item (screened / not, N = 30:
+// 1.03 at 10-80 atoms, 1.07 at 80-150) nor with large molecules (80-150 atoms: one warp 0.99, 2 warps 1.05).
+__host__ __device__ constexpr bool screen_compiled(int maxn, int gt, int g) {
+  return gt == 0 ? g < 8 : gt == 1 && g <= 2 && maxn <= 96;
+}
+
+// Whether a launch screens its alignments of N*N poses, `items` ligand-restarts filling the GPU of `sms` SMs
+// together.  With few poses per warp the estimates and the dealt scoring of the survivors cost more than they save.
+// Measured, screened / not, 10-80 atoms, at N = 12, 16, 20, 24:
+//   FP32, 1, 2, 4 warps: 1.10 0.92 0.80 0.75;  1.25 1.06 0.87 0.79;  1.23 1.12 0.98 0.88
+//   FP16, 1, 2 warps:    1.15 1.08 0.97 0.94;  1.44 1.25 1.08 0.99
+// A large molecule's screening is a long chain, which a GPU with few warps resident cannot hide: 60 ligands of 80-150
+// atoms, 2 warps per item (24 warps per SM) 1.27, 80 ligands (32) 0.89; one warp, 100 ligands (20) 1.13, 150 (30)
+// 0.86.  At 10-80 atoms 41 ligands (16 warps per SM) 0.82.
+inline bool screening_pays(int maxn, int gt, int g, int N, int items, int sms) {
+  if (!screen_compiled(maxn, gt, g)) return false;
+  const int least = gt == 0 ? (g == 1 ? 16 : g == 2 ? 18 : 22) : (g == 1 ? 20 : 24);
+  return N >= least && (maxn <= 96 || (int64_t)items * g >= (int64_t)28 * sms);
+}
+
 constexpr int kScreenKeep = 4;     // best estimates a lane keeps; a lane with more candidates than that falls
                                    // back to scoring all its poses
 constexpr float kScreenMag = 2048.f + kScreenPad;  // 2^11: 12 fraction bits below it in FP32; cell -kScreenPad at 0
