@@ -1217,7 +1217,10 @@ size_t screen_layout(const dock_grid_desc& g, ScreenDev& sc, uint64_t& bias) {
 
 // Quantisation of the field (launch_screen_range's result r): the smallest step with which every corner
 // of every cell fits 7 bits above its cell's base, a multiple of `mult` steps below 16.  False for a
-// field that is flat, or too large or small for the FP32 arithmetic around it.
+// field that is flat, or too large or small for the FP32 arithmetic around it, or whose range is so large against the
+// largest difference within a cell that the base's 4 bits set the step (less than 25 steps for that difference: a large
+// constant on a shallow field), for then the estimates' bound excludes little (500 + sines of amplitude 1: 1.4-1.9
+// times the time of not screening).
 bool screen_steps(const float r[6], bool inside, ScreenDev& sc, float& inv_step) {
   const double vmax = r[0], vmin = -(double)r[1], range = vmax - vmin, spread = r[2];
   const double amax = std::max((double)r[0], (double)r[1]);
@@ -1227,6 +1230,7 @@ bool screen_steps(const float r[6], bool inside, ScreenDev& sc, float& inv_step)
     const double step = std::max(spread / (125.0 - m), range / (125.0 + 15.0 * m));
     if (best == 0 || step < best) best = step, sc.mult = (unsigned)m;
   }
+  if (best > spread / 25.0) return false;
   const float step = (float)(best * 1.0001);
   inv_step = 1.0f / step;
   sc.vmin = (float)vmin;

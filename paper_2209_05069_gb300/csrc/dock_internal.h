@@ -32,6 +32,7 @@ struct ScreenDev {
   float vabs;             // largest |V| in steps
   int inside;             // 1: a boundary voxel is nonzero (the field jumps to 0 at the grid's faces), so
                           // only poses that stay inside the grid may be screened
+  int retry;              // 1: a warp that gave up screening an alignment tries again in the next
 };
 constexpr int kScreenPad = 16;         // cells of padding around the grid: poses that reach past the grid are
                                        // screened without clamping an index

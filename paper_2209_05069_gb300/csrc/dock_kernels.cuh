@@ -585,12 +585,14 @@ __device__ __forceinline__ float3 centre_grid(const float4& cc, const GridK& g) 
 // With early exit and a trilinear grid that has screening cells, the poses are screened first where that pays
 // (dock_screen.cuh) and only those that can hold the best score are scored; the result is the same.  They are
 // then dealt to the item's warps in blocks of kDeal, whether a warp screens them or scores them all (each warp
-// decides for itself), and by single passes otherwise: in blocks of kDeal, 25-64 poses on 4 warps ran 19-23%
-// slower, on 2 warps 13-16%.
+// decides for itself), and by single passes otherwise (blocks of kDeal left warps without poses: 25-64 poses on 4
+// warps ran 19-23% slower).
+// `screen`: cleared where the warp gave up screening, so that the post-alignment does not try again (in launches that
+// fill the GPU many times over; see screening_retries).
 // `scratch` is the warp's bump-pair buffer, unused during an alignment.
 template <int MAXN, int GT, int G, int T>
 __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, const GridK& g, const PocketDev& pk,
-                           bool early_exit, float4* scratch, int wig, int lane, int grp) {
+                           bool early_exit, bool& screen, float4* scratch, int wig, int lane, int grp) {
   if (wig == 0) align_centre(ws, n, lane);
   group_sync<G>(grp);
   const float4 cc = ws.bc;
@@ -608,7 +610,8 @@ __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, 
       // one warp per item: the torsion sweep's records behind the centred pose are free here
       float* buf = G == 1 ? reinterpret_cast<float*>(ws.u.rel + MAXN) : reinterpret_cast<float*>(wig == 0 ? ws.pairs : scratch);
       constexpr int cap = G == 1 ? 6 * MAXN : 4 * PairCap<MAXN>::value;
-      done = screen_align<GT, cap, G>(pk, g, ws.u.rel, n, tab, N, t, mag, wig, buf, lane, best, bidx);
+      if (screen) done = screen_align<GT, cap, G>(pk, g, ws.u.rel, n, tab, N, t, mag, wig, buf, lane, best, bidx);
+      if (!done) screen = pk.screen.retry != 0;
       DOCK_CNT(if (done && lane == 0) for (int f0 = wig * deal; f0 < NN; f0 += G * deal) for (int f = f0; f < min(f0 + deal, NN);
                f += 32 * T) cnt_add(kCntAlignPoses, 32 * T);)
     }
@@ -955,7 +958,8 @@ __device__ void dock_item(ItemSmem<MAXN>& ws, float4* xpairs, const float2* tab_
   if (wig == 0) start_pose(ws, n, bd.ids[l], p.seed, r, pk, lane);
   group_sync<G>(grp);
 
-  const int ai = align_phase<MAXN, GT, G, T>(ws, n, tab_al, p.N, g, pk, p.early_exit != 0, xpairs, wig, lane, grp);
+  bool screen = true;
+  const int ai = align_phase<MAXN, GT, G, T>(ws, n, tab_al, p.N, g, pk, p.early_exit != 0, screen, xpairs, wig, lane, grp);
 
   for (int bi = 0; bi < B; ++bi) {
     const uint32_t ab = __ldg(bd.rot_ab + rb0 + bi);
@@ -970,7 +974,7 @@ __device__ void dock_item(ItemSmem<MAXN>& ws, float4* xpairs, const float2* tab_
     }
   }
 
-  const int pi = p.post_align ? align_phase<MAXN, GT, G, T>(ws, n, tab_al, p.N, g, pk, p.early_exit != 0, xpairs, wig, lane, grp) : -1;
+  const int pi = p.post_align ? align_phase<MAXN, GT, G, T>(ws, n, tab_al, p.N, g, pk, p.early_exit != 0, screen, xpairs, wig, lane, grp) : -1;
   if (wig != 0) return;  // the rest is warp 0's
   const float s = pose_score<MAXN, GT>(ws, n, g, lane);
   const int cc = clash_count<MAXN>(ws, n, bd.excl + (size_t)a0 * kMaskWords, p.dc2, lane);
@@ -1191,6 +1195,7 @@ cudaError_t launch_t(const PocketDev& pk, const BatchDev& b, const ParamsDev& p,
   PocketDev pocket = pk;
   const int together = cfg.together > n_items ? cfg.together : n_items;
   if (!screening_pays(MAXN, GT, G, p.N, together, sms)) pocket.screen.base = nullptr;
+  pocket.screen.retry = screening_retries(together, sms);
   return cudaLaunchKernelEx(&lc, kernel, pocket, b, p, items, n_items, wpb, counter);
 }
 

@@ -47,6 +47,20 @@ inline bool screening_pays(int maxn, int gt, int g, int N, int items, int sms) {
   return N >= least && (maxn <= 96 || (int64_t)items * g >= (int64_t)28 * sms);
 }
 
+// Whether a warp that gave up screening an item's first alignment tries again in its post-alignment.  On a field that
+// screening does not suit it gives up there too; on one that it suits the few items that gave up would run longest, and
+// with less than 100 items per SM the launch waits for them (one warp per item, without: 41-150 ligands 1.15-1.25, 400 small ones 1.04).
+inline int screening_retries(int items, int sms) { return (int64_t)items < (int64_t)100 * sms; }
+
+// Lanes with two candidates after which a warp gives up screening (about 55 candidates in 32 lanes).  On a field whose
+// range is large against the differences between good poses (a large constant, deep repulsion in few places) the
+// bound excludes little: the estimates cost about half of the poses' lookups (FP32 cells; three quarters on FP16) and
+// most poses are then looked up as well.  In the workloads' fields 3-5 of 900 poses are within the bound of the best
+// (98th percentile 22; 50 with large molecules), with repulsion of depth 1000 around 5% of a pocket of depth 1 100
+// (270), in a flat field all.  Time against not screening, 10-80 atoms, without and with giving up (and not trying again,
+// screening_retries): that repulsion, 1,500 ligands, FP32 1.39 -> 1.06, FP16 1.76 -> 1.19, 400 ligands 1.35 -> 1.17 and
+// 1.68 -> 1.44; voxels of -5000 strewn over the workload's field, FP16 1.28 -> 1.03.
+constexpr int kScreenCrowd = 16;
 constexpr int kScreenKeep = 4;     // best estimates a lane keeps; a lane with more candidates than that falls
                                    // back to scoring all its poses
 constexpr float kScreenMag = 2048.f + kScreenPad;  // 2^11: 12 fraction bits below it in FP32; cell -kScreenPad at 0
@@ -193,8 +207,8 @@ __device__ __forceinline__ void screen_score(const GridK& g, const float4* rel, 
 
 // The best of the warp's poses (blocks wig, wig + G, ... of 64), as align_pass over them finds it,
 // left spread over the warp's lanes.  Returns false, with (best, bidx) to be ignored, where screening does
-// not pay: the first block's best estimates per lane span less than two bounds (checked before the rest is
-// estimated), or a lane holds more than kScreenKeep candidates.
+// not pay: after the first, third, ... block of poses more than kScreenCrowd lanes hold two poses within the bound of the best estimate,
+// or in the end a lane holds more than kScreenKeep candidates.
 template <int GT, int CAP, int G>
 __device__ bool screen_align(const PocketDev& pk, const GridK& g, const float4* rel, int n, const float2* tab, int N,
                              const float3& t3, float mag, int wig, float* buf, int lane, float& best, int& bidx) {
@@ -213,6 +227,7 @@ __device__ bool screen_align(const PocketDev& pk, const GridK& g, const float4* 
   // error bound of a pose's estimate in steps, the dropped low bits included
   const float bound = fn * (pk.screen.quant + pk.screen.slope * (4.f / 8192.f + 2.4e-7f * mag) +
                             (fn + 32.f) * 1.1920929e-7f * pk.screen.vabs) + 0.5f;
+  const unsigned slack = __float2uint_ru(bound * kScreenUnits);
   const float3 start = make_float3(t3.x + kScreenMag, t3.y + kScreenMag, t3.z + kScreenMag);
   unsigned top[kScreenKeep + 1];
 #pragma unroll
@@ -227,9 +242,10 @@ __device__ bool screen_align(const PocketDev& pk, const GridK& g, const float4* 
       f += 32;
     }
     if (f < min(f0 + kDeal, NN)) tail = f;
-    if (f0 == wig * kDeal && f0 + 32 <= NN) {
-      const unsigned hi = __reduce_max_sync(kFull, top[0]), lo = __reduce_min_sync(kFull, top[0]);
-      if ((float)(hi - lo) < 2.f * bound * kScreenUnits) return false;
+    if ((f0 / kDeal - wig) / G % 2 == 0) {  // every second block
+      // poses within the bound of the best estimate so far are candidates, as it stands
+      const unsigned hi = __reduce_max_sync(kFull, top[0]);
+      if (__popc(__ballot_sync(kFull, top[1] >= (hi > slack ? hi - slack : 1u))) > kScreenCrowd) return false;
     }
   }
   // the highest estimate's pose, in full
