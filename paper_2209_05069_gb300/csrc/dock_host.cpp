@@ -791,16 +791,21 @@ int launch_batch(dock_ctx* ctx, const PocketDev& pk, char* dev, const Layout& y,
     };
     // The largest molecules first: their items run longest, so the last blocks are short ones (within a bucket items
     // are sorted by cost; 150 ligands of 10-80 atoms 1.4-2.1 times slower with the bulk first, 600 1.05-1.2, 3,000 1.0).
-    // But an SM keeps the carveout of the first kernel it runs, and where the driver chooses, one warp per item at 64
-    // registers (the integer grid, tile 1) takes 32 items of the largest molecules: 211 KB, little L1 for the rest of
-    // the launch.  There the bulk goes first once it is the larger part: 600 ligands 0.88, 3,000 0.50.
-    bool bulk_first = false;
+    // But an SM keeps the carveout of the first kernel it runs.  On the integer grid, whose box L1 holds where it is left
+    // large, the driver's carveout for the largest molecules costs the rest of the launch more than that in full batches:
+    // one warp per item at 64 registers (tile 1) takes 211 KB there (600 ligands with the bulk first 0.88, 3,000 0.50 of
+    // the time), and where most of the work is in molecules above 64 atoms, 0.87-0.92 (2 warps per item, 200-700
+    // large molecules; 152 with few poses 1.3, hence the other line).
+    bool l1_bound = pk.dtype == DOCK_GRID_I16;
+    int bulk = 0, narrow = 0;
     for (int i = 0; i < nb; ++i) {
       const LaunchCfg c = shape(order[i]);
       any_persistent |= c.persistent != 0;
-      bulk_first |= pk.dtype == DOCK_GRID_I16 && c.warps_per_item == 1 && c.tile == 1 && c.smem_carveout < 0;
+      l1_bound &= c.smem_carveout < 0;
+      narrow |= c.warps_per_item == 1 && c.tile == 1;
+      if (plan.bucket_cost[order[i]] > plan.bucket_cost[order[bulk]]) bulk = i;
     }
-    if (bulk_first && total >= (int64_t)100 * ctx->sms)
+    if (l1_bound && ((narrow && total >= (int64_t)100 * ctx->sms) || (nb && order[bulk] > 1 && total >= (int64_t)35 * ctx->sms)))
       std::sort(order, order + nb, [&](int p, int q) { return plan.bucket_cost[p] > plan.bucket_cost[q]; });
     else
       std::reverse(order, order + nb);
