@@ -231,7 +231,11 @@ int dock_resolve_launch(dock_ctx* ctx, int32_t bucket, int64_t items, dock_launc
 /* ---- pocket -------------------------------------------------------------------------------- */
 
 /* Uploads a pocket grid (Section 4.1: the pocket is shared read-only by all ligands) and builds
- * its device layout; the grid stays resident until dock_unload_pocket.  The caller keeps
+ * its device layout; the grid stays resident until dock_unload_pocket.  Device memory: 32 bytes per voxel
+ * (DOCK_GRID_F32), 16 (DOCK_GRID_F16) or 2 per voxel of the nonzero box (DOCK_GRID_I16), and for a trilinear grid
+ * 8 bytes per voxel of the grid widened by 16 voxels on every side (64^3: 6.9 MB) for the rigid alignment's estimates
+ * (dock_params::early_exit).  The latter are left out where they would exceed 16 MiB and twice the former, where all
+ * pockets' together would exceed 1/16 of the device's memory, and for fields that they do not suit.  The caller keeps
  * host_values.  Errors: DOCK_ERR_INVALID (a dimension < 2, spacing <= 0, unknown dtype, a value
  * not finite, or for DOCK_GRID_I16 not an integer in [-32768, 32767]), DOCK_ERR_NOMEM,
  * DOCK_ERR_CUDA. */

@@ -566,6 +566,7 @@ bool same_params(const dock_params& a, const dock_params& b) {
 
 struct Pocket {
   PocketDev dev{};
+  size_t screen_bytes = 0;     // of them the screening cells
   void* cells = nullptr;       // stream-ordered allocation (cudaMallocAsync on the context's stream)
   std::vector<cudaEvent_t> uses;  // recorded after launches that read the pocket, pruned as they finish
   bool closed = false;         // unloaded: unknown to new calls, kept for ligands already submitted
@@ -675,6 +676,7 @@ struct dock_ctx {
   std::string fatal_msg;
   LaunchCfg launch_cfg[kNumBuckets];
   int sms = 0;  // multiprocessors of the device
+  size_t screen_bytes = 0, screen_limit = 0;  // screening cells of the loaded pockets, and how much they may take
   int64_t latency_items = 0;  // serving batches of at most this many items use latency_launch
   int64_t latency_form_ligands = 0;  // serving batches of at most this many ligands: latency form
   uint64_t launch_version = 1;   // bumped by dock_set_launch (invalidates captured graphs)
@@ -763,6 +765,8 @@ void release_pocket(dock_ctx* ctx, Pocket& P) {
   P.uses.clear();
   if (P.cells) cudaFreeAsync(P.cells, ctx->stream);
   P.cells = nullptr;
+  ctx->screen_bytes -= P.screen_bytes;
+  P.screen_bytes = 0;
 }
 
 // The latency-oriented launch shape: one ligand-restart per block of 8 warps, all 8 on it.
@@ -1212,6 +1216,11 @@ void serve_loop(dock_ctx* ctx) {
 
 namespace {
 
+// Bounds on the memory of screening cells, so that pockets and batches that fit without them fit with them but for a
+// small share: all pockets' together 1/kScreenShare of the device's memory; one pocket's twice its own cells, or
+// kScreenSmall (the padding makes them large beside a small or thin grid: 2 x 2 x 1,900 voxels 17 MB beside 61 KB).
+constexpr size_t kScreenShare = 16, kScreenSmall = size_t(16) << 20;
+
 // Layout of a trilinear grid's screening cells: strides and number of cells; cells == 0 where none are
 // built (an axis past the fixed-point coordinates' range, or more than 2^28 cells, 2 GB).  The kernel's
 // index adds 0x45000 (the exponent bits of 2048.f) to each coordinate; the row is lengthened until that
@@ -1289,6 +1298,8 @@ int dock_create(const dock_config* cfg, dock_ctx** out) {
   }
   int sms = 0;
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device);
+  size_t free_bytes = 0, device_bytes = 0;
+  if (e == cudaSuccess) e = cudaMemGetInfo(&free_bytes, &device_bytes);
   void* scratch = nullptr;  // loads the allocation-free entry point's fixed array now, not in a docking call
   if (e == cudaSuccess) e = noalloc_scratch_address(c.device, &scratch);
 #ifdef DOCK_COUNT_WORK
@@ -1300,6 +1311,7 @@ int dock_create(const dock_config* cfg, dock_ctx** out) {
     return DOCK_ERR_CUDA;
   }
   ctx->sms = sms;
+  ctx->screen_limit = device_bytes / kScreenShare;
   ctx->latency_items = c.serve_latency_items < 0 ? 0 : c.serve_latency_items > 0 ? c.serve_latency_items : 2 * 4 * sms;
   ctx->latency_form_ligands = c.serve_latency_form < 0 ? 0 : c.serve_latency_form > 0 ? c.serve_latency_form : 1;
   if (!c.serve_off) ctx->server = std::thread(serve_loop, ctx.get());
@@ -1461,33 +1473,34 @@ int dock_load_pocket(dock_ctx* ctx, const dock_grid_desc* g, const float* host_v
     const size_t cell_bytes = (ncell * (f16 ? 16 : 32) + 255) & ~size_t(255);
     // staging: the voxel values and the field's range
     e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), (nv + 6) * sizeof(float), ctx->stream);
-    unsigned char* cells8 = nullptr;
-    if (e == cudaSuccess && screen_cells) {
-      // the screening cells live behind the pocket's own cells, in one allocation; where that does
-      // not fit the pocket is loaded without them
-      if (cudaMallocAsync(&P.cells, cell_bytes + 8 * screen_cells, ctx->stream) == cudaSuccess) {
-        cells8 = static_cast<unsigned char*>(P.cells) + cell_bytes;
-      } else {
-        cudaGetLastError();
-        P.cells = nullptr;
-      }
-    }
-    if (e == cudaSuccess && !P.cells) e = cudaMallocAsync(&P.cells, cell_bytes, ctx->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(tmp, host_values, nv * sizeof(float), cudaMemcpyHostToDevice, ctx->stream);
-    if (e == cudaSuccess) e = launch_pack_pocket(tmp, P.cells, g->nx, g->ny, g->nz, f16, ctx->stream);
-    if (e == cudaSuccess && cells8) {
+    // The screening cells live behind the pocket's own cells, in one allocation.  They are built for a field that they
+    // suit, within bounds (one pocket's and all pockets' together), and where the allocation succeeds with them.
+    float inv_step = 0.f;
+    bool screened = screen_cells && 8 * screen_cells <= std::max<size_t>(kScreenSmall, 2 * cell_bytes) &&
+                    ctx->screen_bytes + 8 * screen_cells <= ctx->screen_limit;
+    if (e == cudaSuccess && screened) {
       float r[6];
       e = cudaMemsetAsync(tmp + nv, 0, sizeof r, ctx->stream);
       if (e == cudaSuccess)
         e = launch_screen_range(tmp, g->nx, g->ny, g->nz, f16, !inside, reinterpret_cast<int*>(tmp + nv), ctx->stream);
       if (e == cudaSuccess) e = cudaMemcpyAsync(r, tmp + nv, sizeof r, cudaMemcpyDeviceToHost, ctx->stream);
       if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
-      float inv_step = 0.f;
-      if (e == cudaSuccess && screen_steps(r, inside, screen, inv_step)) {
-        e = launch_pack_screen(tmp, cells8, screen, g->nx, g->ny, g->nz, f16, inv_step, ctx->stream);
-        screen.base = reinterpret_cast<const void*>(reinterpret_cast<uintptr_t>(cells8) - 8 * (uintptr_t)screen_bias);
-        P.dev.screen = screen;
-      }
+      screened = e == cudaSuccess && screen_steps(r, inside, screen, inv_step);
+    }
+    if (e == cudaSuccess && screened && cudaMallocAsync(&P.cells, cell_bytes + 8 * screen_cells, ctx->stream) != cudaSuccess) {
+      cudaGetLastError();
+      P.cells = nullptr;
+      screened = false;
+    }
+    if (e == cudaSuccess && !P.cells) e = cudaMallocAsync(&P.cells, cell_bytes, ctx->stream);
+    if (e == cudaSuccess) e = launch_pack_pocket(tmp, P.cells, g->nx, g->ny, g->nz, f16, ctx->stream);
+    if (e == cudaSuccess && screened) {
+      unsigned char* cells8 = static_cast<unsigned char*>(P.cells) + cell_bytes;
+      e = launch_pack_screen(tmp, cells8, screen, g->nx, g->ny, g->nz, f16, inv_step, ctx->stream);
+      screen.base = reinterpret_cast<const void*>(reinterpret_cast<uintptr_t>(cells8) - 8 * (uintptr_t)screen_bias);
+      P.dev.screen = screen;
+      P.screen_bytes = 8 * screen_cells;
     }
     if (tmp) cudaFreeAsync(tmp, ctx->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
@@ -1534,6 +1547,7 @@ int dock_load_pocket(dock_ctx* ctx, const dock_grid_desc* g, const float* host_v
   d.hiy = bhi[1];
   d.hiz = bhi[2];
   const int id = ctx->next_pocket++;
+  ctx->screen_bytes += P.screen_bytes;
   ctx->pockets[id] = P;
   *pocket_id = id;
   return DOCK_OK;
