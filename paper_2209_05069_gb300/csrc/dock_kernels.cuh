@@ -33,7 +33,9 @@
 //    ptxas takes more, and the bound measured 7-15% faster with 2 or 4 warps per item and 19-43% faster
 //    with 8 on databases of 10^2-10^4 ligands.  A register cap (__maxnreg__) in place of the launch bound
 //    generates other code: 64 registers that way made small serving batches (8 warps per item) 8% slower
-//    at the median, so the bound stays.
+//    at the median, so the bound stays.  4 warps per item on FP32 cells hold the screening loop too and spill
+//    more (76 bytes stored, 92 loaded); at 80 registers 1,500 ligands of the uneven mix ran 1.10-1.15 times as long
+//    unscreened and 0.99-1.01 screened (64 -> 80 registers, 8-16 and 24-36 angles per axis), so they stay.
 //  - dock_kernel_mid: 80 registers (3 blocks of 256 threads), 2 warps per item on a trilinear grid.  The
 //    screening loop wants them: 2,000 ligands of the uneven mix 9.5 ms (10.4 at 64, 11.4 at 96), 701 large
 //    molecules 14.6 ms (15.7 and 16.1).
@@ -1180,8 +1182,9 @@ cudaError_t launch_t(const PocketDev& pk, const BatchDev& b, const ParamsDev& p,
     blocks = blocks < resident * sms ? blocks : resident * sms;
     counter = b.next_item + cfg.counter_slot;
   }
-  // the carveout goes with the launch, so that a captured launch keeps its own when another shape of the
-  // same kernel is launched later
+  // A set carveout goes with the launch, so that a captured launch keeps it when another shape of the same kernel is
+  // launched later.  The driver's own choice (-1) is not a value of that attribute; such a launch takes the kernel
+  // function's setting (above).
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3(blocks);
   lc.blockDim = dim3(wpb * 32);
@@ -1189,7 +1192,7 @@ cudaError_t launch_t(const PocketDev& pk, const BatchDev& b, const ParamsDev& p,
   lc.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
-  at[0].val.sharedMemCarveout = cfg.smem_carveout >= 0 ? (unsigned)cfg.smem_carveout : (unsigned)cudaSharedmemCarveoutDefault;
+  at[0].val.sharedMemCarveout = cfg.smem_carveout >= 0 ? (unsigned)cfg.smem_carveout : 0u;
   lc.attrs = at;
   lc.numAttrs = cfg.smem_carveout >= 0 ? 1 : 0;
   PocketDev pocket = pk;
