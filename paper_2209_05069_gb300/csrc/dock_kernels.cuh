@@ -605,7 +605,7 @@ __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, 
   int bidx = 0;  // kept where no pose scores above -infinity (a field past FP16's or FP32's range)
   int deal = 32 * T;  // poses dealt to a warp at a time
   bool done = false;
-  if constexpr (screen_compiled(MAXN, GT, G)) {
+  if constexpr (screen_compiled(GT, G)) {
     float mag;
     if (early_exit && screen_usable(pk, ws.u.rel, n, t, g.inv_h, lane, mag)) {
       deal = kDeal;

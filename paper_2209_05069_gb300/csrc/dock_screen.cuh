@@ -28,9 +28,9 @@ namespace dockgpu {
 // latency counts; a warp has two or three passes then, and the dependent steps of screening cost more than its
 // lookups save (12 ligands in the service 400 us screened, 330 not; 15 large molecules 777 and 673).  On FP16 cells a
 // lookup costs half an FP32 one and screening gains less: nothing with 4 warps per item (screened / not, N = 30:
-// 1.03 at 10-80 atoms, 1.07 at 80-150) nor with large molecules (80-150 atoms: one warp 0.99, 2 warps 1.05).
-__host__ __device__ constexpr bool screen_compiled(int maxn, int gt, int g) {
-  return gt == 0 ? g < 8 : gt == 1 && g <= 2 && maxn <= 96;
+// 1.03 at 10-80 atoms, 1.07 at 80-150).
+__host__ __device__ constexpr bool screen_compiled(int gt, int g) {
+  return gt == 0 ? g < 8 : gt == 1 && g <= 2;
 }
 
 // Whether a launch screens its alignments of N*N poses, `items` ligand-restarts filling the GPU of `sms` SMs
@@ -40,11 +40,12 @@ __host__ __device__ constexpr bool screen_compiled(int maxn, int gt, int g) {
 //   FP16, 1, 2 warps:    1.15 1.08 0.97 0.94;  1.44 1.25 1.08 0.99
 // A large molecule's screening is a long chain, which a GPU with few warps resident cannot hide: 60 ligands of 80-150
 // atoms, 2 warps per item (24 warps per SM) 1.27, 80 ligands (32) 0.89; one warp, 100 ligands (20) 1.13, 150 (30)
-// 0.86.  At 10-80 atoms 41 ligands (16 warps per SM) 0.82.
+// 0.86; 4 warps, 41 ligands (32) 1.09, 60 (47) 0.91.  At 10-80 atoms 41 ligands (16 warps per SM) 0.82.  (FP16, 2 warps, full GPU: 501 large molecules 0.96 on a
+// 96^3 grid, 1.05 on 64^3, whose cells stay closer; both ways below the time before the screening.)
 inline bool screening_pays(int maxn, int gt, int g, int N, int items, int sms) {
-  if (!screen_compiled(maxn, gt, g)) return false;
+  if (!screen_compiled(gt, g)) return false;
   const int least = gt == 0 ? (g == 1 ? 16 : g == 2 ? 18 : 22) : (g == 1 ? 20 : 24);
-  return N >= least && (maxn <= 96 || (int64_t)items * g >= (int64_t)28 * sms);
+  return N >= least && (maxn <= 96 || (int64_t)items * g >= (int64_t)(g == 4 ? 40 : 28) * sms);
 }
 
 // Whether a warp that gave up screening an item's first alignment tries again in its post-alignment.  On a field that

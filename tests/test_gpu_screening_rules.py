@@ -56,9 +56,11 @@ def _sized(n_atoms, count):
 
 
 @pytest.mark.parametrize("grid,shape,atoms,ligands,screened", [
-    # 28 warps per SM of 152: 4,256 one-warp items, 2,128 of two warps
+    # 28 warps per SM of 152: 4,256 one-warp items, 2,128 of two warps; with 4 warps 40: 1,520
     ("f32", ONE, 110, 430, True), ("f32", ONE, 110, 420, False), ("f32", TWO, 110, 215, True), ("f32", TWO, 110, 210, False),
-    ("f32", ONE, 90, 20, True), ("f16", TWO, 90, 20, True), ("f16", TWO, 110, 430, False), ("f16", ONE, 110, 430, False)])
+    ("f32", FOUR, 110, 155, True), ("f32", FOUR, 110, 150, False),
+    ("f32", ONE, 90, 20, True), ("f16", TWO, 90, 20, True),
+    ("f16", TWO, 110, 215, True), ("f16", TWO, 110, 210, False), ("f16", ONE, 110, 430, True), ("f16", ONE, 110, 420, False)])
 def test_large_molecules_need_a_full_gpu(grid, shape, atoms, ligands, screened):
     import torch
     if torch.cuda.get_device_properties(0).multi_processor_count != 152:
