@@ -645,7 +645,7 @@ __device__ int align_phase(ItemSmem<MAXN>& ws, int n, const float2* tab, int N, 
 __host__ __device__ constexpr int bump_tile(int gt, int g) { return gt == 1 && g == 4 ? 2 : 4; }
 
 template <int kBumpTile>
-__device__ __forceinline__ unsigned check_pairs(const float4* pairs, int cnt, const float2* tab, int A, int nq,
+__device__ __forceinline__ unsigned bump_loop(const float4* pairs, int cnt, const float2* tab, int A, int nq,
                                                 float dc2, bool early_exit, unsigned prior, int lane) {
   __syncwarp();
   unsigned bits = 0;
@@ -688,6 +688,17 @@ __device__ __forceinline__ unsigned check_pairs(const float4* pairs, int cnt, co
   }
   __syncwarp();
   return bits;
+}
+
+// The check with an item's tile.  Up to 32 angles have a single pass, which 8 warps per item (there the check's latency
+// counts) run without the three empty ones: 16 and 32 angles 2-5% faster, other counts the same.  In the kernels of 1 to
+// 4 warps the second loop costs more than that (4,003 ligands 2-8% slower at 256 angles), and so did a loop for each
+// remainder of 4 in all of them.
+template <int GT, int G>
+__device__ __forceinline__ unsigned check_pairs(const float4* pairs, int cnt, const float2* tab, int A, int nq,
+                                                float dc2, bool early_exit, unsigned prior, int lane) {
+  if (G == 8 && nq == 1) return bump_loop<1>(pairs, cnt, tab, A, nq, dc2, early_exit, prior, lane);
+  return bump_loop<bump_tile(GT, G)>(pairs, cnt, tab, A, nq, dc2, early_exit, prior, lane);
 }
 
 // Sweeps rotatable bond (a, b): angles theta_k = 2 pi k / A about the axis a -> b through b move
@@ -787,13 +798,13 @@ __device__ int torsion_phase(ItemSmem<MAXN>& ws, int n, int a, int b, const uint
       const unsigned bal = __ballot_sync(kFull, act);
       const int na = __popc(bal);
       if (cnt + na > CAP) {
-        clash_bits |= check_pairs<bump_tile(GT, G)>(pairs, cnt, tab, A, nq, dc2, early_exit, clash_bits, lane);
+        clash_bits |= check_pairs<GT, G>(pairs, cnt, tab, A, nq, dc2, early_exit, clash_bits, lane);
         cnt = 0;
       }
       if (act) pairs[cnt + __popc(bal & lt)] = make_float4(C, Pa, Pb, 0.f);
       cnt += na;
     }
-    clash_bits |= check_pairs<bump_tile(GT, G)>(pairs, cnt, tab, A, nq, dc2, early_exit, clash_bits, lane);
+    clash_bits |= check_pairs<GT, G>(pairs, cnt, tab, A, nq, dc2, early_exit, clash_bits, lane);
     if (!split)
       ws.clash[lane] = clash_bits;
     else if (clash_bits)
