@@ -38,6 +38,10 @@ FP32_PEAK_TFLOPS = SM_COUNT * FP32_LANES * 2 * SM_MAX_GHZ / 1e3
 # 7 linear interpolations (a subtract and a multiply-add each), 1 accumulate.
 FLOPS_ALIGN, FLOPS_TORSION, FLOPS_FINAL = 18 + 3 + 21 + 1, 12 + 3 + 21 + 1, 6 + 3 + 21 + 1
 
+# L1 data-pipe wavefronts per warp-wide load in the 33-64-atom kernels (ncu, profiles/dock_screening.md): an alignment
+# estimate from 8-byte screening cells, and a lookup by grid type (FP32 32-byte cell, FP16 16-byte cell, int16 voxel).
+WAVEFRONTS_ESTIMATE, WAVEFRONTS_LOOKUP = 11.5, {0: 23.1, 1: 15.4, 2: 2.8}
+
 
 def parse():
     ap = argparse.ArgumentParser()
@@ -235,6 +239,13 @@ def executed_work(dock, local, pk, grid_dtype, db, prm, bucket, tuning):
         c = cctx.exec_counters(reset=True)
         cctx.batch_destroy(b)
     return c
+
+
+def kernel_entry(gt, g, tile):
+    """The docking kernel's entry point for a grid type, warps per item and pose tile (their register budgets differ)."""
+    if g == 1 and not (gt == 2 and tile == 1):
+        return "dock_kernel_wide"
+    return "dock_kernel_mid" if gt != 2 and g == 2 else "dock_kernel"
 
 
 def launch_fields(table):
@@ -811,43 +822,43 @@ def main():
     bytes_per_lookup = {"f16": 16, "i16": 2}.get(grid_dtype, 32)
     gt = {"f16": 1, "i16": 2}.get(grid_dtype, 0)
     sh = ctx.resolve_launch(dom["bucket"], dom["ligands"] * w.restarts)
-    entry = "dock_kernel_wide" if gt == 0 and sh["warps_per_item"] == 1 else "dock_kernel"
+    entry = kernel_entry(gt, sh["warps_per_item"], sh["pose_tile"])
     kernel = f"{entry}<{32 * (dom['bucket'] + 1)}, {gt}, {sh['warps_per_item']}, {sh['pose_tile']}>"
     launch_s = dom["ms_per_launch"] / 1e3
-    # the L1 data pipe's roof at the SM clock measured during the timed steps: one wavefront per SM
-    # per clock, and a scattered 32-byte sector (one FP32 corner-packed cell) takes one wavefront
+    # the L1 data pipe's roof at the SM clock measured during the timed steps: one wavefront per SM per clock
     sm_ghz = (clk["sm_mhz"] / 1e3) if clk and clk.get("sm_mhz") else SM_MAX_GHZ
-    peak_gbs = SM_COUNT * sm_ghz * 32
+    peak_waves = SM_COUNT * sm_ghz * 1e9
     algo_gbs = dom["lookups_per_launch"] * bytes_per_lookup / launch_s / 1e9
     executed = None if args.no_counters else executed_work(dock, local, pk, grid_dtype, db, prm, dom["bucket"], tuning)
     scattered_gbs = gather_peak * bytes_per_lookup / 1e9
     path_gbs = lookups * bytes_per_lookup / mean_s / 1e9
     if executed:
-        achieved = executed["sectors"] * 32 / launch_s / 1e9
-        frac_note = ("executed: the launch's distinct 32-byte sectors (counted per warp-wide load by the counter "
-                     "build on the same ligands and shapes) x 32 B / mean launch time.  The model (one data-pipe "
-                     "wavefront per sector) fits scattered 32-byte cells (FP32; ncu's data-pipe utilisation on this "
-                     "kernel agrees); on FP16 and int16 grids neighbouring lanes share lines, a wavefront serves "
-                     "several sectors, the figure can exceed 1 and those kernels are issue-bound (see profiles)")
+        est = max(executed["loads"] - executed["lookups"], 0)   # the alignment's estimates are loads, not lookups
+        waves = (est * WAVEFRONTS_ESTIMATE + (executed["loads"] - est) * WAVEFRONTS_LOOKUP[gt]) / 32
+        achieved = waves / launch_s
+        frac_note = (f"executed loads of the launch (counter build, same ligands and shapes) / 32 lanes x the data-pipe "
+                     f"wavefronts that ncu counts per warp-wide load ({WAVEFRONTS_ESTIMATE} for an 8-byte estimate, "
+                     f"{WAVEFRONTS_LOOKUP[gt]} for this grid's lookup; profiles/dock_screening.md) / mean launch time.  Shared-memory "
+                     "wavefronts (about 6% of the pipe) are not in it, and no unit is saturated: the same profile has the issue "
+                     "rates, which bound the integer grid")
     else:
-        achieved = algo_gbs
-        frac_note = "algorithmic lookups x bytes per lookup / mean launch time (no counter pass)"
-    roofline = {"bound": "l1tex", "kernel": kernel, "achieved": achieved, "peak": peak_gbs, "unit": "GB/s",
-                "frac": achieved / peak_gbs, "achieved_source": frac_note,
+        achieved = dom["lookups_per_launch"] / 32 * WAVEFRONTS_LOOKUP[gt] / launch_s
+        frac_note = "algorithmic lookups x wavefronts per lookup / mean launch time (no counter pass)"
+    roofline = {"bound": "l1tex", "kernel": kernel, "achieved": achieved / 1e9, "peak": peak_waves / 1e9,
+                "unit": "G wavefronts/s", "frac": achieved / peak_waves, "achieved_source": frac_note,
                 "traffic": committed_kernel_traffic(grid_dtype, kernel, db, dom["bucket"], dom["ligands"]),
-                "peak_source": f"derived: L1 data pipe, one 32-byte sector (wavefront) per SM per clock, "
-                               f"{SM_COUNT} SMs x {sm_ghz:.3f} GHz (median SM clock of the timed steps) x 32 B",
+                "peak_source": f"derived: L1 data pipe, one wavefront per SM per clock, {SM_COUNT} SMs x {sm_ghz:.3f} GHz "
+                               f"(median SM clock of the timed steps)",
                 "launch_ms": dom["ms_per_launch"], "launch_ligands": dom["ligands"],
-                "executed": dict(executed, loads_per_lookup=executed["loads"] / max(executed["lookups"], 1),
+                "executed": dict(executed, estimates=est, wavefronts=waves,
                                  sectors_per_load=executed["sectors"] / max(executed["loads"], 1),
                                  lines_per_load=executed["lines"] / max(executed["loads"], 1),
-                                 lookups_per_s=executed["lookups"] / launch_s,
-                                 sectors_per_s=executed["sectors"] / launch_s,
-                                 line_frac=executed["lines"] / launch_s / (SM_COUNT * sm_ghz * 1e9))
+                                 lookups_per_s=executed["lookups"] / launch_s, estimates_per_s=est / launch_s)
                 if executed else None,
                 "algorithmic": {"lookups_per_launch": dom["lookups_per_launch"], "bytes_per_lookup": bytes_per_lookup,
-                                "achieved": algo_gbs, "frac": algo_gbs / peak_gbs,
-                                "note": "every angle of every bond scored, every lookup one cell of bytes_per_lookup"},
+                                "achieved": algo_gbs, "unit": "GB/s",
+                                "note": "what scoring every pose and every angle in full would read, one cell of "
+                                        "bytes_per_lookup per lookup, in the launch's time"},
                 "scattered_gather": {"achieved": scattered_gbs, "lookups_per_s": gather_peak,
                                      "algorithmic_over_scattered": algo_gbs / scattered_gbs,
                                      "source": "measured in this run by dock_gather_peak: the same lookups at "

@@ -225,7 +225,8 @@ constexpr float kRound = 12582912.0f;  // 1.5 * 2^23: kRound + q has unit spacin
 // low mantissa bits (exact for 0 <= u < 2^23), and one fused add-and-min per axis turns the bits into a
 // box-relative index clamped to the far border: an index past the box lands there, and so does a
 // coordinate that is negative (its sum's bits fall below 2^23's and wrap), beyond 2^23 or not a number;
-// the border is zero.  The FMA pipe does the rounding, which as a conversion took the conversion pipe.
+// the border is zero.  The FMA pipe does the rounding, which as a conversion took the conversion pipe.  (Past voxel 2^23
+// of a longer stored box, where coordinates are a voxel apart or more, it is some voxel of the box.)
 __device__ __forceinline__ unsigned voxel_index(float u, int hi) {
   return __viaddmin_u32(__float_as_uint(__fadd_rd(u, 8388608.f)), 0u - 0x4B000000u, (unsigned)hi);
 }
