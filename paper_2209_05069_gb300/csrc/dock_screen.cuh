@@ -40,8 +40,9 @@ __host__ __device__ constexpr bool screen_compiled(int gt, int g) {
 //   FP16, 1, 2 warps:    1.15 1.08 0.97 0.94;  1.44 1.25 1.08 0.99
 // A large molecule's screening is a long chain, which a GPU with few warps resident cannot hide: 60 ligands of 80-150
 // atoms, 2 warps per item (24 warps per SM) 1.27, 80 ligands (32) 0.89; one warp, 100 ligands (20) 1.13, 150 (30)
-// 0.86; 4 warps, 41 ligands (32) 1.09, 60 (47) 0.91.  At 10-80 atoms 41 ligands (16 warps per SM) 0.82.  (FP16, 2 warps, full GPU: 501 large molecules 0.96 on a
-// 96^3 grid, 1.05 on 64^3, whose cells stay closer; both ways below the time before the screening.)
+// 0.86; 4 warps, 41 ligands (32) 1.09, 60 (47) 0.91.  At 10-80 atoms 41 ligands (16 warps per SM) 0.82.  (FP16, 2 warps,
+// full GPU: 501 large molecules 0.96 on a 96^3 grid, 1.05 on 64^3, whose cells stay closer; both ways below the time
+// before the screening.)
 inline bool screening_pays(int maxn, int gt, int g, int N, int items, int sms) {
   if (!screen_compiled(gt, g)) return false;
   const int least = gt == 0 ? (g == 1 ? 16 : g == 2 ? 18 : 22) : (g == 1 ? 20 : 24);
@@ -50,7 +51,8 @@ inline bool screening_pays(int maxn, int gt, int g, int N, int items, int sms) {
 
 // Whether a warp that gave up screening an item's first alignment tries again in its post-alignment.  On a field that
 // screening does not suit it gives up there too; on one that it suits the few items that gave up would run longest, and
-// with less than 100 items per SM the launch waits for them (one warp per item, without: 41-150 ligands 1.15-1.25, 400 small ones 1.04).
+// with less than 100 items per SM the launch waits for them (one warp per item, without: 41-150 ligands 1.15-1.25, 400
+// small ones 1.04).
 inline int screening_retries(int items, int sms) { return (int64_t)items < (int64_t)100 * sms; }
 
 // Lanes with two candidates after which a warp gives up screening (about 55 candidates in 32 lanes).  On a field whose
@@ -208,8 +210,8 @@ __device__ __forceinline__ void screen_score(const GridK& g, const float4* rel, 
 
 // The best of the warp's poses (blocks wig, wig + G, ... of 64), as align_pass over them finds it,
 // left spread over the warp's lanes.  Returns false, with (best, bidx) to be ignored, where screening does
-// not pay: after the first, third, ... block of poses more than kScreenCrowd lanes hold two poses within the bound of the best estimate,
-// or in the end a lane holds more than kScreenKeep candidates.
+// not pay: after the first, third, ... block of poses more than kScreenCrowd lanes hold two poses within the bound of
+// the best estimate, or in the end a lane holds more than kScreenKeep candidates.
 template <int GT, int CAP, int G>
 __device__ bool screen_align(const PocketDev& pk, const GridK& g, const float4* rel, int n, const float2* tab, int N,
                              const float3& t3, float mag, int wig, float* buf, int lane, float& best, int& bidx) {
