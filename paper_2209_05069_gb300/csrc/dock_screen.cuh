@@ -38,15 +38,16 @@ __host__ __device__ constexpr bool screen_compiled(int gt, int g) {
 // Measured, screened / not, 10-80 atoms, at N = 12, 16, 20, 24:
 //   FP32, 1, 2, 4 warps: 1.10 0.92 0.80 0.75;  1.25 1.06 0.87 0.79;  1.23 1.12 0.98 0.88
 //   FP16, 1, 2 warps:    1.15 1.08 0.97 0.94;  1.44 1.25 1.08 0.99
-// A large molecule's screening is a long chain, which a GPU with few warps resident cannot hide: 60 ligands of 80-150
-// atoms, 2 warps per item (24 warps per SM) 1.27, 80 ligands (32) 0.89; one warp, 100 ligands (20) 1.13, 150 (30)
-// 0.86; 4 warps, 41 ligands (32) 1.09, 60 (47) 0.91.  At 10-80 atoms 41 ligands (16 warps per SM) 0.82.  (FP16, 2 warps,
-// full GPU: 501 large molecules 0.96 on a 96^3 grid, 1.05 on 64^3, whose cells stay closer; both ways below the time
-// before the screening.)
+// A large molecule's screening is a long chain, which a GPU with few warps resident cannot hide.  80-150 atoms: 60 ligands
+// with 2 warps per item (24 warps per SM) 1.27, 80 ligands (32) 0.89; one warp, 100 ligands (20) 1.13, 150 (30) 0.86; 4
+// warps, 41 ligands (32) 1.09, 60 (47) 0.91.  10-80 atoms, where the 65-96-atom bucket decides: less than 8 warps per SM
+// one warp per item 1.16 (FP16 1.18), 4 warps 1.10, but 2 warps 0.82-0.98.  (FP16, 2 warps, full GPU: 501 large molecules
+// 0.96 on a 96^3 grid, 1.05 on 64^3, whose cells stay closer; both ways below the time before the screening.)
 inline bool screening_pays(int maxn, int gt, int g, int N, int items, int sms) {
   if (!screen_compiled(gt, g)) return false;
   const int least = gt == 0 ? (g == 1 ? 16 : g == 2 ? 18 : 22) : (g == 1 ? 20 : 24);
-  return N >= least && (maxn <= 96 || (int64_t)items * g >= (int64_t)(g == 4 ? 40 : 28) * sms);
+  const int warps = maxn <= 64 ? 0 : maxn <= 96 ? (g == 2 ? 0 : 8) : g == 4 ? 40 : 28;  // per SM
+  return N >= least && (int64_t)items * g >= (int64_t)warps * sms;
 }
 
 // Whether a warp that gave up screening an item's first alignment tries again in its post-alignment.  On a field that

@@ -59,7 +59,9 @@ def _sized(n_atoms, count):
     # 28 warps per SM of 152: 4,256 one-warp items, 2,128 of two warps; with 4 warps 40: 1,520
     ("f32", ONE, 110, 430, True), ("f32", ONE, 110, 420, False), ("f32", TWO, 110, 215, True), ("f32", TWO, 110, 210, False),
     ("f32", FOUR, 110, 155, True), ("f32", FOUR, 110, 150, False),
-    ("f32", ONE, 90, 20, True), ("f16", TWO, 90, 20, True),
+    # up to 96 atoms 8 with 1 and 4 warps: 1,216 and 304 items, none with 2
+    ("f32", ONE, 90, 125, True), ("f32", ONE, 90, 118, False), ("f32", FOUR, 90, 32, True), ("f32", FOUR, 90, 29, False),
+    ("f16", ONE, 90, 118, False), ("f16", TWO, 90, 4, True), ("f32", ONE, 60, 4, True),
     ("f16", TWO, 110, 215, True), ("f16", TWO, 110, 210, False), ("f16", ONE, 110, 430, True), ("f16", ONE, 110, 420, False)])
 def test_large_molecules_need_a_full_gpu(grid, shape, atoms, ligands, screened):
     import torch
