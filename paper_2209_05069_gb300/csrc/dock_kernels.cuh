@@ -1210,7 +1210,7 @@ cudaError_t launch_t(const PocketDev& pk, const BatchDev& b, const ParamsDev& p,
   PocketDev pocket = pk;
   const int together = cfg.together > n_items ? cfg.together : n_items;
   if (!screening_pays(MAXN, GT, G, p.N, together, sms)) pocket.screen.base = nullptr;
-  pocket.screen.retry = screening_retries(together, sms);
+  pocket.screen.retry = screening_retries(G, together, sms);
   return cudaLaunchKernelEx(&lc, kernel, pocket, b, p, items, n_items, wpb, counter);
 }
 

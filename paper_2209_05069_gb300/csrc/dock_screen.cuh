@@ -52,9 +52,10 @@ inline bool screening_pays(int maxn, int gt, int g, int N, int items, int sms) {
 
 // Whether a warp that gave up screening an item's first alignment tries again in its post-alignment.  On a field that
 // screening does not suit it gives up there too; on one that it suits the few items that gave up would run longest, and
-// with less than 100 items per SM the launch waits for them (one warp per item, without: 41-150 ligands 1.15-1.25, 400
-// small ones 1.04).
-inline int screening_retries(int items, int sms) { return (int64_t)items < (int64_t)100 * sms; }
+// with one warp per item and less than 100 items per SM the launch waits for them (without a second try: 41-150 ligands
+// 1.15-1.25, 400 small ones 1.04); with more warps an item's share is shorter and that shows below 30 only (100 ligands
+// 1.05).
+inline int screening_retries(int g, int items, int sms) { return (int64_t)items < (int64_t)(g == 1 ? 100 : 30) * sms; }
 
 // Lanes with two candidates after which a warp gives up screening (about 55 candidates in 32 lanes).  On a field whose
 // range is large against the differences between good poses (a large constant, deep repulsion in few places) the
